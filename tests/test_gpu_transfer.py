@@ -1,0 +1,56 @@
+"""Canonical array <-> field on the GPU (tiles of sites through shared memory): every count of
+elements per site, ragged tiles, pads and arrays that are only 8-byte aligned, bit for bit."""
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+SEED = synth.SEED_BASE + 41
+
+
+@pytest.fixture(scope="module")
+def su3s(gpu_lib):
+    return gpu_lib
+
+
+def in_field_order(x, f):
+    """Canonical (V, nmu, ncomp, 2) values in the field's order, pads zero."""
+    v, nmu, nc, _ = x.shape
+    n = f.tensor.numel() // (nmu * nc * 2)
+    p = torch.zeros((n, nmu, nc, 2), dtype=x.dtype, device=x.device)
+    p[:v] = x
+    b = f.block if f.block else n
+    return p.view(n // b, b, nmu, nc, 2).permute(0, 2, 3, 1, 4).reshape(-1)
+
+
+@pytest.mark.parametrize("layout,block", [(0, 0), (1, 4), (1, 32), (1, 1024)])
+@pytest.mark.parametrize("kind,nmu", [("matrix", 1), ("matrix", 3), ("matrix", 4), ("matrix", 8),
+                                      ("vector", 1), ("vector", 4), ("real", 1), ("real", 3)])
+@pytest.mark.parametrize("dims", [(1, 1, 1, 1), (31, 1, 1, 1), (4, 4, 2, 1), (11, 3, 1, 1),
+                                  (257, 1, 1, 1), (7, 5, 3, 4)])
+def test_tiles_are_exact(su3s, dims, kind, nmu, layout, block):
+    lat = su3s.Lattice(dims)
+    K = {"matrix": su3s.MATRIX, "vector": su3s.VECTOR, "real": su3s.REAL}[kind]
+    f = su3s.Field(lat, K, nmu, su3s.F64, layout, block or 64)
+    n = int(np.prod(f.canonical_shape))
+    g = torch.Generator(device="cuda").manual_seed(7)
+    buf = torch.randn(n + 1, dtype=torch.float64, device="cuda", generator=g)
+    for off in (0, 1):   # 16-byte aligned, and 8-byte aligned only
+        x = buf[off:off + n].view(f.canonical_shape)
+        f.tensor.fill_(float("nan"))
+        f.pack(x)
+        w = {"matrix": 9, "vector": 3}.get(kind)
+        if w:
+            assert torch.equal(f.tensor, in_field_order(x.reshape(-1, nmu, w, 2), f))
+        assert torch.equal(f.unpack(), x)
+        out = torch.full((n + 2,), 5.0, dtype=torch.float64, device="cuda")
+        rc = su3s.load().su3s_field_unpack(f._h, ctypes.c_void_p(out[off:].data_ptr()),
+                                           ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == 0
+        assert torch.equal(out[off:off + n], x.reshape(-1))
+        assert out[n + off:].eq(5.0).all() and out[:off].eq(5.0).all()
