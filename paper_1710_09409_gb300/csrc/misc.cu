@@ -78,6 +78,185 @@ int check_redot(const su3s_field* x, const su3s_field* y, const double* out) {
 }
 
 // ------------------------------------------------------------ reunitarise
+// The 9 elements of a stored matrix, and back.
+template <int PREC>
+__device__ __forceinline__ void reunit_load(const FieldDesc& f, int64_t b, double* r) {
+#pragma unroll
+  for (int c = 0; c < 9; ++c) {
+    const double2 v = get_complex<PREC>(f.ptr, b + c * f.s_c);
+    r[2 * c] = v.x;
+    r[2 * c + 1] = v.y;
+  }
+}
+template <int PREC>
+__device__ __forceinline__ void reunit_store(const FieldDesc& f, int64_t b, const double* r) {
+#pragma unroll
+  for (int c = 0; c < 9; ++c) put_complex<PREC>(f.ptr, b + c * f.s_c, r[2 * c], r[2 * c + 1]);
+}
+
+// Projection of one matrix (rows r[0..5], r[6..11], r[12..17]) by the
+// definition: Gram-Schmidt over rows, two sweeps, then division by the
+// principal cube root of the determinant's phase.  Out of line and from the
+// field itself: it serves the matrices whose norms leave the range in which
+// reunit_fast is the same projection (see there).
+template <int PREC>
+__device__ __noinline__ void reunit_sweeps(const FieldDesc& src, const FieldDesc& dst, int64_t bs,
+                                           int64_t bd) {
+  double r[18];
+  reunit_load<PREC>(src, bs, r);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+#pragma unroll
+    for (int rep = 0; rep < 2; ++rep)
+#pragma unroll
+      for (int p = 0; p < i; ++p) {
+        double cr = 0.0, ci = 0.0;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const double pr = r[6 * p + 2 * j], pi = r[6 * p + 2 * j + 1];
+          const double xr = r[6 * i + 2 * j], xi = r[6 * i + 2 * j + 1];
+          cr += pr * xr + pi * xi;
+          ci += pr * xi - pi * xr;
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const double pr = r[6 * p + 2 * j], pi = r[6 * p + 2 * j + 1];
+          r[6 * i + 2 * j] -= cr * pr - ci * pi;
+          r[6 * i + 2 * j + 1] -= cr * pi + ci * pr;
+        }
+      }
+    double nn = 0.0;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) nn += r[6 * i + j] * r[6 * i + j];
+    const double inv = rsqrt(nn);
+#pragma unroll
+    for (int j = 0; j < 6; ++j) r[6 * i + j] *= inv;
+  }
+  double dr = 0.0, di = 0.0;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const int a = (j + 1) % 3, b = (j + 2) % 3;
+    const double xr = r[6 + 2 * a] * r[12 + 2 * b] - r[6 + 2 * a + 1] * r[12 + 2 * b + 1] -
+                      (r[6 + 2 * b] * r[12 + 2 * a] - r[6 + 2 * b + 1] * r[12 + 2 * a + 1]);
+    const double xi = r[6 + 2 * a] * r[12 + 2 * b + 1] + r[6 + 2 * a + 1] * r[12 + 2 * b] -
+                      (r[6 + 2 * b] * r[12 + 2 * a + 1] + r[6 + 2 * b + 1] * r[12 + 2 * a]);
+    dr += r[2 * j] * xr - r[2 * j + 1] * xi;
+    di += r[2 * j] * xi + r[2 * j + 1] * xr;
+  }
+  const double phi = atan2(di, dr);
+  double sn, cs;
+  sincos(-phi / 3.0, &sn, &cs);
+#pragma unroll
+  for (int c = 0; c < 9; ++c) {
+    const double re = r[2 * c], im = r[2 * c + 1];
+    r[2 * c] = cs * re - sn * im;
+    r[2 * c + 1] = cs * im + sn * re;
+  }
+  reunit_store<PREC>(dst, bd, r);
+}
+
+// a = b times c, complex
+__device__ __forceinline__ void zmul(double& ar, double& ai, double br, double bi, double cr,
+                                     double ci) {
+  const double re = fma(br, cr, -(bi * ci));
+  ai = fma(br, ci, bi * cr);
+  ar = re;
+}
+
+// The same projection with fewer FP64 operations (the FP64 pipe bounds the
+// kernel: 91% busy; 2.59 M FP64 matrices 1,989 -> 1,024 us against the sweeps
+// and FP64 atan2 and sincos of the definition, which stay for the cases below;
+// errors against extended precision, near-unitary input: 4.6e-17 rms, 3.9e-16
+// at most, the definition's 4.3e-17 and 3.2e-16).  Rows 0 and 1 as in the definition.  Of row 2 only a phase is free:
+// orthonormal to rows 0 and 1 it is e^{i alpha} w, w = conj(r0 x r1), so
+// Gram-Schmidt's two sweeps and normalisation come down to the direction of
+// d = <w, row 2>, and e^{i alpha} = d/|d| is also the determinant.  Dividing by
+// its principal cube root leaves rows 0, 1 times q and w times conj(q)^2,
+// q = e^{-i alpha/3}.  q is formed in FP32 (atan2f, sincosf: the branch of
+// the cube root is that of the signs of d) and refined by one step on q^3 d/|d|
+// = 1: with q^3 d/|d| = 1 + z, |z| < 1e-6, q (1 - z/3 + 2/9 z^2) is exact to
+// z^3 < 1e-18.  Returns false where a norm is NaN, zero, or so large or small
+// that it could overflow or underflow here and not in the definition.
+__device__ __forceinline__ bool reunit_fast(double* r) {
+  double* a = r;  // rows 0 and 1, not normalised until the end
+  double* b = r + 6;
+  double n0 = 0.0;
+#pragma unroll
+  for (int j = 0; j < 6; ++j) n0 = fma(a[j], a[j], n0);
+  const double inv0 = rsqrt(n0);
+  const double rn0 = inv0 * inv0;
+#pragma unroll
+  for (int rep = 0; rep < 2; ++rep) {
+    double cr = 0.0, ci = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      cr = fma(a[2 * j], b[2 * j], fma(a[2 * j + 1], b[2 * j + 1], cr));
+      ci = fma(a[2 * j], b[2 * j + 1], fma(-a[2 * j + 1], b[2 * j], ci));
+    }
+    cr *= rn0;
+    ci *= rn0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      b[2 * j] = fma(-cr, a[2 * j], fma(ci, a[2 * j + 1], b[2 * j]));
+      b[2 * j + 1] = fma(-cr, a[2 * j + 1], fma(-ci, a[2 * j], b[2 * j + 1]));
+    }
+  }
+  double n1 = 0.0;
+#pragma unroll
+  for (int j = 0; j < 6; ++j) n1 = fma(b[j], b[j], n1);
+  const double inv1 = rsqrt(n1);
+  // x = a x b; d = sum_j x_j row2_j
+  double x[6], dr = 0.0, di = 0.0;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const int k = (j + 1) % 3, l = (j + 2) % 3;
+    x[2 * j] = fma(a[2 * k], b[2 * l], fma(-a[2 * k + 1], b[2 * l + 1],
+               fma(-a[2 * l], b[2 * k], a[2 * l + 1] * b[2 * k + 1])));
+    x[2 * j + 1] = fma(a[2 * k], b[2 * l + 1], fma(a[2 * k + 1], b[2 * l],
+                   fma(-a[2 * l], b[2 * k + 1], -(a[2 * l + 1] * b[2 * k]))));
+    dr = fma(x[2 * j], r[12 + 2 * j], fma(-x[2 * j + 1], r[12 + 2 * j + 1], dr));
+    di = fma(x[2 * j], r[12 + 2 * j + 1], fma(x[2 * j + 1], r[12 + 2 * j], di));
+  }
+  const double nd = fma(dr, dr, di * di);
+  const double invd = rsqrt(nd);
+  if (!(n0 > 0x1p-200 && n0 < 0x1p200 && n1 > 0x1p-200 && n1 < 0x1p200 && nd > 0x1p-800 &&
+        nd < 0x1p800))
+    return false;
+  const double er = dr * invd, ei = di * invd;
+  float qs, qc;
+  sincosf(atan2f(__double2float_rn(ei), __double2float_rn(er)) * (-1.0f / 3.0f), &qs, &qc);
+  const double tr = (double)qc, ti = (double)qs;
+  double sr, si, zr, zi;
+  zmul(sr, si, tr, ti, tr, ti);
+  zmul(zr, zi, sr, si, tr, ti);
+  sr = fma(zr, er, fma(-zi, ei, -1.0));
+  si = fma(zr, ei, zi * er);
+  // 1 - z/3 + 2/9 z^2 = 1 + z (2/9 z - 1/3)
+  zmul(zr, zi, sr, si, fma(sr, 2.0 / 9.0, -1.0 / 3.0), si * (2.0 / 9.0));
+  const double qr = fma(tr, zr, fma(-ti, zi, tr)), qi = fma(tr, zi, fma(ti, zr, ti));
+  // rows 0, 1: q times the normalised rows; row 2: e^{i alpha} q conj(x) / |x|,
+  // the conjugate of x times conj(e^{i alpha} q) / |x|
+  double n2 = 0.0;
+#pragma unroll
+  for (int j = 0; j < 6; ++j) n2 = fma(x[j], x[j], n2);
+  const double inv2 = rsqrt(n2);
+  const double pr = fma(er, qr, -(ei * qi)), pi = -fma(er, qi, ei * qr);
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    a[j] *= inv0;
+    b[j] *= inv1;
+    x[j] *= inv2;
+  }
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    zmul(r[2 * j], r[2 * j + 1], a[2 * j], a[2 * j + 1], qr, qi);
+    zmul(r[6 + 2 * j], r[6 + 2 * j + 1], b[2 * j], b[2 * j + 1], qr, qi);
+    zmul(r[12 + 2 * j], r[12 + 2 * j + 1], x[2 * j], x[2 * j + 1], pr, pi);
+    r[12 + 2 * j + 1] = -r[12 + 2 * j + 1];
+  }
+  return true;
+}
+
 template <int PREC>
 __global__ void __launch_bounds__(256) k_reunit(FieldDesc src, FieldDesc dst, int64_t V, int nmu) {
   const int64_t n = V * nmu;
@@ -87,59 +266,9 @@ __global__ void __launch_bounds__(256) k_reunit(FieldDesc src, FieldDesc dst, in
     const int64_t s = q - (int64_t)mu * V;
     const int64_t bs = fbase(src, s, mu), bd = fbase(dst, s, mu);
     double r[18];
-#pragma unroll
-    for (int c = 0; c < 9; ++c) {
-      double2 v = get_complex<PREC>(src.ptr, bs + c * src.s_c);
-      r[2 * c] = v.x;
-      r[2 * c + 1] = v.y;
-    }
-    // Gram-Schmidt over rows, two projection sweeps
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-#pragma unroll
-      for (int rep = 0; rep < 2; ++rep)
-#pragma unroll
-        for (int p = 0; p < i; ++p) {
-          double cr = 0.0, ci = 0.0;
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            const double pr = r[6 * p + 2 * j], pi = r[6 * p + 2 * j + 1];
-            const double xr = r[6 * i + 2 * j], xi = r[6 * i + 2 * j + 1];
-            cr += pr * xr + pi * xi;
-            ci += pr * xi - pi * xr;
-          }
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            const double pr = r[6 * p + 2 * j], pi = r[6 * p + 2 * j + 1];
-            r[6 * i + 2 * j] -= cr * pr - ci * pi;
-            r[6 * i + 2 * j + 1] -= cr * pi + ci * pr;
-          }
-        }
-      double nn = 0.0;
-#pragma unroll
-      for (int j = 0; j < 6; ++j) nn += r[6 * i + j] * r[6 * i + j];
-      const double inv = rsqrt(nn);
-#pragma unroll
-      for (int j = 0; j < 6; ++j) r[6 * i + j] *= inv;
-    }
-    double dr = 0.0, di = 0.0;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const int a = (j + 1) % 3, b = (j + 2) % 3;
-      const double xr = r[6 + 2 * a] * r[12 + 2 * b] - r[6 + 2 * a + 1] * r[12 + 2 * b + 1] -
-                        (r[6 + 2 * b] * r[12 + 2 * a] - r[6 + 2 * b + 1] * r[12 + 2 * a + 1]);
-      const double xi = r[6 + 2 * a] * r[12 + 2 * b + 1] + r[6 + 2 * a + 1] * r[12 + 2 * b] -
-                        (r[6 + 2 * b] * r[12 + 2 * a + 1] + r[6 + 2 * b + 1] * r[12 + 2 * a]);
-      dr += r[2 * j] * xr - r[2 * j + 1] * xi;
-      di += r[2 * j] * xi + r[2 * j + 1] * xr;
-    }
-    const double phi = atan2(di, dr);
-    double sn, cs;
-    sincos(-phi / 3.0, &sn, &cs);
-#pragma unroll
-    for (int c = 0; c < 9; ++c)
-      put_complex<PREC>(dst.ptr, bd + c * dst.s_c, cs * r[2 * c] - sn * r[2 * c + 1],
-                        cs * r[2 * c + 1] + sn * r[2 * c]);
+    reunit_load<PREC>(src, bs, r);
+    if (reunit_fast(r)) reunit_store<PREC>(dst, bd, r);
+    else reunit_sweeps<PREC>(src, dst, bs, bd);
   }
 }
 

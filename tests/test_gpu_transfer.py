@@ -1,11 +1,13 @@
 """Canonical array <-> field on the GPU (tiles of sites through shared memory): every count of
-elements per site, ragged tiles, pads and arrays that are only 8-byte aligned, bit for bit."""
+elements per site, ragged tiles, pads and arrays that are only 8-byte aligned, bit for bit; and
+the projection to SU(3) at the edges of its fast path, against the CPU oracle."""
 import ctypes
 
 import numpy as np
 import pytest
 import torch
 
+import oracle
 import synth
 
 pytestmark = pytest.mark.gpu
@@ -54,3 +56,35 @@ def test_tiles_are_exact(su3s, dims, kind, nmu, layout, block):
         assert rc == 0
         assert torch.equal(out[off:off + n], x.reshape(-1))
         assert out[n + off:].eq(5.0).all() and out[:off].eq(5.0).all()
+
+
+def test_projection_at_the_edges_of_the_fast_path(su3s):
+    """Scales whose squares overflow or vanish, negative real determinants (the cube root's branch
+    cut), nearly dependent rows, and matrices without a projection (zero, NaN)."""
+    n = 64
+    u = synth.su3(SEED, 0, n) + 0.05 * synth.gauss_matrix(SEED, 1, n)
+    q = np.linalg.qr(np.random.default_rng(3).standard_normal((n, 3, 3)))[0]
+    q *= -np.sign(np.linalg.det(q))[:, None, None]          # real, determinant -1
+    real = np.stack([q, np.zeros_like(q)], -1)
+    close = u.copy()
+    close[:, 1] = close[:, 0] + 1e-3 * close[:, 1]
+    cases = {"unit": u, "2^120": u * 2.0 ** 120, "2^-120": u * 2.0 ** -120, "2^480": u * 2.0 ** 480,
+             "2^-480": u * 2.0 ** -480, "det -1": real, "close rows": close}
+    lat = su3s.Lattice((4, 4, 4, 1))
+    for name, x in cases.items():
+        f = su3s.Field(lat)
+        f.upload(x)
+        su3s.reunitarize(f, f)                              # in place
+        # rows 1e-3 apart: the rounding of the inputs' difference, times 1e3
+        tol = 1e-12 if name == "close rows" else 1e-14
+        assert np.abs(f.download() - oracle.reunitarize(x)).max() < tol, name
+    x = u.copy()
+    x[5] = 0.0
+    x[9, 2, 1, 0] = np.nan
+    f = su3s.Field(lat)
+    f.upload(x)
+    su3s.reunitarize(f, f)
+    got, ref = f.download(), oracle.reunitarize(x)
+    assert np.array_equal(np.isnan(got).any((1, 2, 3)), np.isnan(ref).any((1, 2, 3)))
+    fine = ~np.isnan(ref).any((1, 2, 3))
+    assert np.abs(got - ref)[fine].max() < 1e-14
