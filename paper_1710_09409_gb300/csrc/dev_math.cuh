@@ -203,7 +203,6 @@ struct MathDF {
   static constexpr bool kScaled = false;
   static constexpr bool kPaired = true;   // complex products in packed (re, im) lanes
   static constexpr bool kGuard = true;    // FP32 exponent range: sites are range-checked
-  static constexpr bool kPackSplit = true;  // complex inputs split, outputs converted, in pairs
   __device__ static __forceinline__ R from_bits(uint32_t lo, uint32_t hi) {
     return df_split_bits(lo, hi);
   }
@@ -291,15 +290,6 @@ struct MathDF {
 // instructions save.  Results are identical to MathDF's.
 struct MathDFScalar : MathDF {
   static constexpr bool kPaired = false;
-};
-
-// The same arithmetic with every FP64 input split and every output converted
-// one real at a time (MathDF packs the two reals of a complex element: the
-// same values).  Measured faster for the Wilson term, whose schedule lost more
-// to the packed operations' register pairs than the packing saved (48^4:
-// 1,923 against 1,887 GB/s).
-struct MathDFUnpacked : MathDF {
-  static constexpr bool kPackSplit = false;
 };
 
 // --------------------------------------------- MathDF, packed (re, im) lanes
@@ -647,11 +637,10 @@ __device__ __forceinline__ void df2_to_double(const DAcc2& a, double& d0, double
   d1 = df_assemble(s.y, e.y);
 }
 
-// Whether M splits and converts complex elements in packed pairs.
+// Whether M splits and converts complex elements in packed pairs (the pair arithmetic).
 template <class M>
 __host__ __device__ constexpr bool pack_split() {
-  if constexpr (std::is_base_of<MathDF, M>::value) return M::kPackSplit;
-  else return false;
+  return std::is_base_of<MathDF, M>::value;
 }
 
 // One complex element (16 bytes: re lo, re hi, im lo, im hi) into the

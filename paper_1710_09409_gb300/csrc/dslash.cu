@@ -44,8 +44,7 @@ struct Phase {
 
 template <class M>
 __device__ __forceinline__ typename M::A neg_acc(const typename M::A& a) {
-  if constexpr (std::is_same<typename M::A, DAcc>::value) return DAcc{-a.S, -a.lo};
-  else if constexpr (std::is_same<typename M::A, FAcc>::value) return FAcc{-a.hh, -a.cr, a.e};
+  if constexpr (std::is_same<typename M::A, FAcc>::value) return FAcc{-a.hh, -a.cr, a.e};
   else return -a;
 }
 
@@ -53,31 +52,6 @@ __device__ __forceinline__ typename M::A neg_acc(const typename M::A& a) {
 template <class M>
 __device__ __forceinline__ void half_spinor(typename M::R* h, const typename M::R* u,
                                             const typename M::R* l, Phase P) {
-  if constexpr (M::kPaired) {
-    // the pair arithmetic: real and imaginary parts in packed lanes, each lane
-    // repeating MathDF::add's operations (the copy, then TwoSum of the
-    // leading parts with the tail gathered)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const df a = P.swap ? l[2 * c + 1] : l[2 * c];
-      const df b = P.swap ? l[2 * c] : l[2 * c + 1];
-      const float2 S = make_float2(u[2 * c].h, u[2 * c + 1].h);
-      const float2 lo = make_float2(u[2 * c].l, u[2 * c + 1].l);
-      const float2 xh = make_float2(P.neg_re ? -a.h : a.h, P.neg_im ? -b.h : b.h);
-      const float2 xl = make_float2(P.neg_re ? -a.l : a.l, P.neg_im ? -b.l : b.l);
-      const float2 s = f2_add(S, xh);
-      const float2 nbp = f2_sub(S, s);          // -bp
-      const float2 ap = f2_add(s, nbp);         // s - bp
-      const float2 db = f2_add(xh, nbp);        // xh - bp
-      const float2 da = f2_sub(S, ap);
-      float2 t = f2_add(da, db);
-      t = f2_add(t, xl);
-      const float2 lo2 = f2_add(lo, t);
-      h[2 * c] = df_norm(s.x, lo2.x);
-      h[2 * c + 1] = df_norm(s.y, lo2.y);
-    }
-    return;
-  }
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const typename M::R a = P.swap ? l[2 * c + 1] : l[2 * c];
@@ -95,20 +69,6 @@ __device__ __forceinline__ void half_spinor(typename M::R* h, const typename M::
 // out += P chi for a colour vector of accumulators.
 template <class M>
 __device__ __forceinline__ void add_rebuilt(typename M::A* out, const typename M::A* chi, Phase P) {
-  if constexpr (M::kPaired) {
-    // real and imaginary parts combined in packed lanes (MathDF::combine per lane)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const DAcc a = P.swap ? chi[2 * c + 1] : chi[2 * c];
-      const DAcc b = P.swap ? chi[2 * c] : chi[2 * c + 1];
-      DAcc2 o = dacc2_get(out[2 * c], out[2 * c + 1]);
-      const DAcc2 x{make_float2(P.neg_re ? -a.S : a.S, P.neg_im ? -b.S : b.S),
-                    make_float2(P.neg_re ? -a.lo : a.lo, P.neg_im ? -b.lo : b.lo)};
-      df2_combine<1>(o, x);
-      dacc2_put(out[2 * c], out[2 * c + 1], o);
-    }
-    return;
-  }
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const typename M::A a = P.swap ? chi[2 * c + 1] : chi[2 * c];
@@ -215,6 +175,7 @@ __device__ __noinline__ void dslash_site_f64(const FieldDesc& dst, const FieldDe
 // loads' latency is hidden behind a term's arithmetic without holding the
 // next operands in registers.  Slots are [element][thread], 16 bytes each.
 constexpr int kDslashElems = 21;
+constexpr int kDslashThreads = 128;
 
 // Issue the copies of term t (direction t >> 1, backward if t is odd) of site s.
 __device__ __forceinline__ void stage_term(uint4* slot, int nt, const FieldDesc& U,
@@ -350,29 +311,343 @@ __device__ __forceinline__ void dslash_staged(const FieldDesc& dst, const FieldD
   cp_async_wait_all();
 }
 
-// One thread per site, a grid of one wave (the neighbours of the sites in
-// flight stay in the L2 cache), each thread with 21 staging slots.
+// Native FP64 and fixed point: one thread per site, each with 21 staging slots.
 template <class M>
-__global__ void __launch_bounds__(128) k_dslash(FieldDesc dst, FieldDesc U, FieldDesc psi, LatGeo g) {
+__global__ void __launch_bounds__(kDslashThreads) k_dslash(FieldDesc dst, FieldDesc U, FieldDesc psi, LatGeo g) {
   extern __shared__ __align__(16) uint4 d_slots[];
   dslash_staged<M>(dst, U, psi, g, (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
                    (int64_t)gridDim.x * blockDim.x, d_slots + threadIdx.x, (int)blockDim.x);
+}
+
+// ------------------------------------- pair arithmetic: both spins of h per lane pair
+// The pair arithmetic has a kernel of its own, bound by instruction issue and
+// the FMA pipe (62% busy, issue 62%), not by memory.  It packs every FP32
+// operation over the two components k = 0, 1 of the half spinor (the two lanes
+// of f32x2): both are multiplied by the same link element, so the link's reals
+// are duplicated and nothing else is swapped or negated (packing (re, im) of
+// one output instead needs swapped copies of h and signed copies of the link).
+//   - Phases ride along as +-1 factors of packed FMAs.  Directions go in the
+//     order x, y, t, z; s_mu has the entries i f_k (x, z) or f_k (y, t), so
+//     h_k = u_k + f_k (i) l, where the factor i only exchanges the addresses of
+//     l's real and imaginary parts, and the lower accumulators hold the lower
+//     spins (times i for x, z) in the lane order of the direction's columns;
+//     they are turned where that changes, three times per site.
+//   - The projections are formed in FP64 (one DFMA per real on a pipe that is
+//     idle otherwise): only the 12 reals of h are split into pairs, not the 24
+//     of the spinor, and h enters rounded to nearest.
+//   - Operands come one colour at a time (two spins of u, two of l, three link
+//     elements).  The next colour is read and split, work of the ALU pipe,
+//     between the products of the current one, work of the FMA pipe; each
+//     colour's slots are refilled for the next term as soon as they are read.
+// Measured at 32^3 x 64 (pair arithmetic, default launch): 1,031 us before (one
+// (re, im) pair per lane pair, 242 registers, 10,870 instructions per site),
+// 884 us with the spins packed, 787 with the colours pipelined (8,580
+// instructions), 755 with four waves of blocks, 740 with walked addresses.
+// Not kept: tiles of sites in 2, 3 or 4 dimensions per block with and without
+// L1 (863-880 against 873 us), 128 registers (815), the first term opening the
+// accumulators (761 against 755).
+
+// a += f * b lane-wise (MathDF::combine with a sign per lane: f = +-1, so every
+// product is exact)
+__device__ __forceinline__ void dp_combine_sign(dpa& a, const dpa& b, float2 f) {
+  const float2 s = f2_fma(b.S, f, a.S);
+  const float2 nbp = f2_sub(a.S, s);
+  const float2 ap = f2_add(s, nbp);
+  const float2 db = f2_fma(b.S, f, nbp);
+  const float2 da = f2_sub(a.S, ap);
+  float2 t = f2_add(da, db);
+  t = f2_fma(b.lo, f, t);
+  a.S = s;
+  a.lo = f2_add(a.lo, t);
+}
+
+__device__ __forceinline__ void dp_swap_lanes(dpa& a) {
+  a.S = make_float2(a.S.y, a.S.x);
+  a.lo = make_float2(a.lo.y, a.lo.x);
+}
+
+// One real of the half spinors k = 0, 1 into pairs, the leading part rounded to
+// nearest (the split truncates), which halves the trailing part the products
+// round with.  The range guard takes h's words instead of the spinor's: NaN and
+// infinities reach h, and large components that cancel leave an h that FP64
+// holds and the pairs can represent.
+__device__ __forceinline__ dp dslash_half(double x0, double x1, uint32_t& gm) {
+  const uint32_t h0 = (uint32_t)__double2hiint(x0), h1 = (uint32_t)__double2hiint(x1);
+  gm = guard_max(gm, h0, h1);
+  const dp a = dp_split((uint32_t)__double2loint(x0), h0, (uint32_t)__double2loint(x1), h1);
+  const float2 h = f2_add(a.h, a.l);
+  return dp{h, f2_sub(a.l, f2_sub(h, a.h))};
+}
+
+// Offsets of the 8 neighbours of a site, from its coordinates.
+struct Coords {
+  int32_t x[4];
+};
+__device__ __forceinline__ Coords site_coords(const LatGeo& g, int64_t s) {
+  Coords c;
+  uint32_t q = (uint32_t)s;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const uint32_t r = q / (uint32_t)g.L[d];
+    c.x[d] = (int32_t)(q - r * (uint32_t)g.L[d]);
+    q = r;
+  }
+  c.x[3] = (int32_t)q;
+  return c;
+}
+__device__ __forceinline__ int32_t neighbour(const LatGeo& g, const Coords& c, int32_t s, int mu,
+                                             bool bwd) {
+  const int32_t st = mu == 0 ? 1 : mu == 1 ? g.stride[1] : mu == 2 ? g.stride[2] : g.stride[3];
+  const int32_t L = mu == 0 ? g.L[0] : mu == 1 ? g.L[1] : mu == 2 ? g.L[2] : g.L[3];
+  const int32_t x = mu == 0 ? c.x[0] : mu == 1 ? c.x[1] : mu == 2 ? c.x[2] : c.x[3];
+  const int32_t wrap = (L - 1) * st;
+  return bwd ? (x == 0 ? s + wrap : s - st) : (x == L - 1 ? s - wrap : s + st);
+}
+
+// Direction of position t >> 1 in the order x, y, t, z.
+__device__ __forceinline__ int dir_at(int t) {
+  const int p = t >> 1;
+  return p < 2 ? p : 5 - p;
+}
+
+// Where one term's operands lie: the neighbour spinor's and the link's first
+// elements.
+struct TermSrc {
+  const uint4* psi;
+  const uint4* U;
+};
+__device__ __forceinline__ TermSrc term_src(const FieldDesc& U, const FieldDesc& psi, const LatGeo& g,
+                                            const Coords& c, int32_t s, int t) {
+  const int mu = dir_at(t);
+  const bool bwd = (t & 1) != 0;
+  const int32_t n = neighbour(g, c, s, mu, bwd);
+  return TermSrc{reinterpret_cast<const uint4*>(psi.ptr) + elem_base(psi, n, 0),
+                 reinterpret_cast<const uint4*>(U.ptr) + elem_base(U, bwd ? n : s, mu)};
+}
+
+// Stage colour j of a term: the four spin components and the link's column j
+// (backward: row j).  Slots: [colour][4 spins, 3 link elements][thread].
+__device__ __forceinline__ void stage_colour(uint4* slot, const TermSrc& src, const FieldDesc& U,
+                                             const FieldDesc& psi, bool bwd, int j) {
+  const uint4* p = src.psi + j * psi.s_c;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    cp_async16(slot + (7 * j + k) * kDslashThreads, p);
+    p += psi.s_mu;
+  }
+  const int64_t step = bwd ? U.s_c : 3 * U.s_c;
+  p = src.U + (bwd ? 3 * j : j) * U.s_c;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    cp_async16(slot + (7 * j + 4 + i) * kDslashThreads, p);
+    p += step;
+  }
+  cp_async_commit();
+}
+
+// One colour's operands in pairs: h_k of that colour (lanes k = 0, 1) and the
+// link's three elements (lanes re, im).
+struct ColourOps {
+  dp hr, hm;
+  df2 u[3];
+};
+
+// How a term reads its operands (uniform across the grid).
+struct TermForm {
+  int l0, l1;           // byte offsets of the spin components added to u_0 and u_1
+  int flip;             // 8: real and imaginary parts of l exchanged (factor i)
+  uint32_t r0, r1, i0, i1;  // high words of the +-1.0 factors
+  uint32_t neg;         // sign flip of the link's imaginary parts (adjoint)
+};
+__device__ __forceinline__ TermForm term_form(int t) {
+  const int mu = dir_at(t);
+  const bool bwd = (t & 1) != 0;
+  const bool im = (mu & 1) == 0, sw = mu < 2;
+  const bool p0 = (mu != 1) == bwd, p1 = (mu != 2) == bwd;  // f_k = +1
+  TermForm f;
+  f.l0 = (sw ? 3 : 2) * kDslashThreads * 16;
+  f.l1 = (sw ? 2 : 3) * kDslashThreads * 16;
+  f.flip = im ? 8 : 0;
+  f.i0 = p0 ? 0x3FF00000u : 0xBFF00000u;
+  f.i1 = p1 ? 0x3FF00000u : 0xBFF00000u;
+  f.r0 = p0 != im ? 0x3FF00000u : 0xBFF00000u;
+  f.r1 = p1 != im ? 0x3FF00000u : 0xBFF00000u;
+  f.neg = bwd ? 0x80000000u : 0u;
+  return f;
+}
+
+// h_k = u_k + f_k (i) l of colour j: with the factor i the real part takes
+// -im(l) and the imaginary part re(l).
+__device__ __forceinline__ void read_half(ColourOps& o, const uint4* slot, const TermForm& f, int j,
+                                          uint32_t& gm) {
+  const unsigned char* base = reinterpret_cast<const unsigned char*>(slot + 7 * j * kDslashThreads);
+  const double2 u0 = *reinterpret_cast<const double2*>(base);
+  const double2 u1 = *reinterpret_cast<const double2*>(base + kDslashThreads * 16);
+  const double a0 = *reinterpret_cast<const double*>(base + f.l0 + f.flip);
+  const double b0 = *reinterpret_cast<const double*>(base + f.l0 + (8 - f.flip));
+  const double a1 = *reinterpret_cast<const double*>(base + f.l1 + f.flip);
+  const double b1 = *reinterpret_cast<const double*>(base + f.l1 + (8 - f.flip));
+  o.hr = dslash_half(fma(a0, __hiloint2double((int)f.r0, 0), u0.x),
+                     fma(a1, __hiloint2double((int)f.r1, 0), u1.x), gm);
+  o.hm = dslash_half(fma(b0, __hiloint2double((int)f.i0, 0), u0.y),
+                     fma(b1, __hiloint2double((int)f.i1, 0), u1.y), gm);
+}
+__device__ __forceinline__ void read_link_elem(ColourOps& o, const uint4* slot, const TermForm& f, int j,
+                                               int i, uint32_t& gm) {
+  const uint4 v = slot[(7 * j + 4 + i) * kDslashThreads];
+  gm = guard_max(gm, v.y, v.w);
+  o.u[i] = df2_split(v.x, v.y, v.z, v.w ^ f.neg);
+}
+
+__global__ void __launch_bounds__(kDslashThreads, 3)
+    k_dslash_df(const __grid_constant__ FieldDesc dst, const __grid_constant__ FieldDesc U,
+                const __grid_constant__ FieldDesc psi, const __grid_constant__ LatGeo g) {
+  extern __shared__ __align__(16) uint4 d_slots[];
+  uint4* slot = d_slots + threadIdx.x;
+  const int32_t V = (int32_t)g.V;
+  const int64_t stride = (int64_t)gridDim.x * kDslashThreads;
+  int64_t s = (int64_t)blockIdx.x * kDslashThreads + threadIdx.x;
+  if (s >= V) return;
+  Coords co = site_coords(g, s);
+  uint32_t gm = 0, gm_next = 0;
+  ColourOps cur;
+  {
+    const TermSrc src = term_src(U, psi, g, co, (int32_t)s, 0);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) stage_colour(slot, src, U, psi, false, j);
+    cp_async_wait<2>();
+    const TermForm f = term_form(0);
+    read_half(cur, slot, f, 0, gm_next);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) read_link_elem(cur, slot, f, 0, i, gm_next);
+  }
+  for (;;) {
+    const int64_t sn = s + stride;
+    dpa up[6], low[6];   // [2 colour + re/im]
+#pragma unroll
+    for (int r = 0; r < 6; ++r) {
+      up[r] = dpa{make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+      low[r] = up[r];
+    }
+    gm = 0;
+#pragma unroll 1
+    for (int t = 0; t < 8; ++t) {
+      // this term's first colour was read during the term before (at t = 0 the
+      // previous site's last): its range guard counts from here
+      gm = max(gm, gm_next);
+      gm_next = 0;
+      // where the next term's operands come from (past the last site: this
+      // site again, read and not used)
+      if (t == 7 && sn < V) co = site_coords(g, sn);
+      const int tn = (t + 1) & 7;
+      const bool bwd_n = (tn & 1) != 0;
+      const TermSrc src = term_src(U, psi, g, co, (int32_t)(t == 7 && sn < V ? sn : s), tn);
+      const TermForm fc = term_form(t), fn = term_form(tn);
+      dpa re[3], im[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        // colour j is in registers: refill its slots with the next term's, and
+        // read colour j + 1 (after the last, the next term's first)
+        ColourOps nxt;
+        stage_colour(slot, src, U, psi, bwd_n, j);
+        cp_async_wait<2>();
+        const int jn = j < 2 ? j + 1 : 0;
+        const TermForm& fr = j < 2 ? fc : fn;
+        uint32_t& gr = j < 2 ? gm : gm_next;
+        read_half(nxt, slot, fr, jn, gr);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          const df2& e = cur.u[i];
+          const dp er{make_float2(e.h.x, e.h.x), make_float2(e.l.x, e.l.x)};
+          const dp em{make_float2(e.h.y, e.h.y), make_float2(e.l.y, e.l.y)};
+          if (j == 0) dp_cterm<true, 1, false, false>(re[i], im[i], er, em, cur.hr, cur.hm);
+          else dp_cterm<false, 1, false, false>(re[i], im[i], er, em, cur.hr, cur.hm);
+          read_link_elem(nxt, slot, fr, jn, i, gr);
+        }
+        cur = nxt;
+      }
+      const float2 f = make_float2(__uint_as_float((fc.i0 & 0x80000000u) | 0x3F800000u),
+                                   __uint_as_float((fc.i1 & 0x80000000u) | 0x3F800000u));
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        df2_combine<1>(up[2 * i], re[i]);
+        df2_combine<1>(up[2 * i + 1], im[i]);
+        dp_combine_sign(low[2 * i], re[i], f);
+        dp_combine_sign(low[2 * i + 1], im[i], f);
+      }
+      // lower accumulators: x holds i * lower in lanes (3, 2); y lower in lanes
+      // (3, 2); t lower in lanes (2, 3); z i * lower in lanes (2, 3)
+      if (t == 3) {
+#pragma unroll
+        for (int r = 0; r < 6; ++r) dp_swap_lanes(low[r]);
+      } else if (t == 1 || t == 5) {
+        // x -> y: lower = -i (i lower); t -> z: i lower
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const dpa a = low[2 * c], b = low[2 * c + 1];
+          const dpa na{f2_neg(a.S), f2_neg(a.lo)}, nb{f2_neg(b.S), f2_neg(b.lo)};
+          low[2 * c] = t == 1 ? b : nb;
+          low[2 * c + 1] = t == 1 ? na : a;
+        }
+      }
+    }
+    if (gm >= guard_hi(2)) {
+      dslash_site_f64<MathF64>(dst, U, psi, g, s);
+    } else {
+      const int64_t b = elem_base(dst, s, 0);
+      char* p = reinterpret_cast<char*>(dst.ptr);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const int64_t e = b + c * dst.s_c;
+        pair_store_c(p, e, e + dst.s_mu, true, up[2 * c], up[2 * c + 1]);
+        // lower = -i (i lower)
+        const dpa n{f2_neg(low[2 * c].S), f2_neg(low[2 * c].lo)};
+        pair_store_c(p, e + 2 * dst.s_mu, e + 3 * dst.s_mu, true, low[2 * c + 1], n);
+      }
+    }
+    if (sn >= V) break;
+    s = sn;
+  }
+  cp_async_wait_all();
+}
+
+// `waves` waves of blocks, the threads' sites strided by the grid.
+static cudaError_t dslash_grid(const void* kernel, size_t smem, int64_t V, int waves, dim3* grid) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int per_sm = 1;
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kDslashThreads, smem);
+  if (e != cudaSuccess) return e;
+  const int64_t nb = (int64_t)(per_sm > 0 ? per_sm : 1) * sm_count() * waves;
+  const int64_t need = (V + kDslashThreads - 1) / kDslashThreads;
+  *grid = dim3((unsigned)(nb < need ? nb : need));
+  return cudaSuccess;
+}
+
+static cudaError_t launch_dslash_df(const su3s_field* dest, const su3s_field* U, const su3s_field* psi,
+                                    cudaStream_t st) {
+  const LatGeo g = lat_geo(psi);
+  const size_t smem = (size_t)kDslashElems * 16 * kDslashThreads;
+  dim3 grid;
+  // four waves: blocks do not all take the same time, and what one finishes
+  // early the next ones use (one wave 787 us, two 769, four 755, one site per
+  // thread 766 at 32^3 x 64)
+  const cudaError_t e = dslash_grid((const void*)k_dslash_df, smem, g.V, 4, &grid);
+  if (e != cudaSuccess) return e;
+  k_dslash_df<<<grid, kDslashThreads, smem, st>>>(dest->desc, U->desc, psi->desc, g);
+  return cudaGetLastError();
 }
 
 template <class M>
 static cudaError_t launch_dslash(const su3s_field* dest, const su3s_field* U, const su3s_field* psi,
                                  cudaStream_t st) {
   const LatGeo g = lat_geo(psi);
-  const size_t smem = (size_t)kDslashElems * 16 * 128;
-  cudaError_t e = cudaFuncSetAttribute(k_dslash<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  int per_sm = 1;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dslash<M>, 128, smem);
+  const size_t smem = (size_t)kDslashElems * 16 * kDslashThreads;
+  dim3 grid;
+  // one wave: the neighbours of the sites in flight stay in the L2 cache
+  const cudaError_t e = dslash_grid((const void*)k_dslash<M>, smem, g.V, 1, &grid);
   if (e != cudaSuccess) return e;
-  int64_t nb = (int64_t)(per_sm > 0 ? per_sm : 1) * sm_count();   // one wave
-  const int64_t need = (g.V + 127) / 128;
-  const dim3 grid((unsigned)(nb < need ? nb : need));
-  k_dslash<M><<<grid, 128, smem, st>>>(dest->desc, U->desc, psi->desc, g);
+  k_dslash<M><<<grid, kDslashThreads, smem, st>>>(dest->desc, U->desc, psi->desc, g);
   return cudaGetLastError();
 }
 
@@ -399,7 +674,7 @@ SU3S_EXPORT int su3s_dslash(su3s_field* dest, const su3s_field* U, const su3s_fi
   if (psi->V == 0) return SU3S_OK;
   cudaError_t ce = m == MATH_F64  ? launch_dslash<MathF64>(dest, U, psi, st)
                    : m == MATH_FX ? launch_dslash<MathFX>(dest, U, psi, st)
-                                  : launch_dslash<MathDFUnpacked>(dest, U, psi, st);
+                                  : launch_dslash_df(dest, U, psi, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "Wilson hopping-term kernel launch");
   return SU3S_OK;
 }
