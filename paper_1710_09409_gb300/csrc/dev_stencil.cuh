@@ -77,14 +77,32 @@ __device__ __forceinline__ int64_t shift_site_rt(const LatGeo& g, int64_t s, int
   return s + (int64_t)(c2 - c) * st;
 }
 
-// One thread per site; the grid is one wave, so the sites in flight (and the
-// backward links and neighbours they share) fit the L2 cache, and the loop over
-// the 8 terms is rolled.  Colour matrices: the terms run through a single
-// product routine (the backward link's adjoint is taken in its load), which
-// keeps the matrix-product code small enough for the instruction cache (+29%
-// at 48^4 over separate forward and backward routines).  Colour vectors: the
-// matrix-vector code is small, and separate forward and backward routines,
-// with the first term opening the accumulators, are faster (+13%).
+// A site's coordinates, and its neighbours from them (one division per
+// coordinate and site instead of two per neighbour).
+struct Coords {
+  int32_t x[4];
+};
+__device__ __forceinline__ Coords site_coords(const LatGeo& g, int64_t s) {
+  Coords c;
+  uint32_t q = (uint32_t)s;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const uint32_t r = q / (uint32_t)g.L[d];
+    c.x[d] = (int32_t)(q - r * (uint32_t)g.L[d]);
+    q = r;
+  }
+  c.x[3] = (int32_t)q;
+  return c;
+}
+__device__ __forceinline__ int32_t neighbour(const LatGeo& g, const Coords& c, int32_t s, int mu,
+                                             bool bwd) {
+  const int32_t st = mu == 0 ? 1 : mu == 1 ? g.stride[1] : mu == 2 ? g.stride[2] : g.stride[3];
+  const int32_t L = mu == 0 ? g.L[0] : mu == 1 ? g.L[1] : mu == 2 ? g.L[2] : g.L[3];
+  const int32_t x = mu == 0 ? c.x[0] : mu == 1 ? c.x[1] : mu == 2 ? c.x[2] : c.x[3];
+  const int32_t wrap = (L - 1) * st;
+  return bwd ? (x == 0 ? s + wrap : s - st) : (x == L - 1 ? s - wrap : s + st);
+}
+
 // Asynchronous 16-byte copies global -> shared (cp.async), used to stage the
 // next term's operands of a stencil while the current term is computed.
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {

@@ -379,31 +379,6 @@ __device__ __forceinline__ dp dslash_half(double x0, double x1, uint32_t& gm) {
   return dp{h, f2_sub(a.l, f2_sub(h, a.h))};
 }
 
-// Offsets of the 8 neighbours of a site, from its coordinates.
-struct Coords {
-  int32_t x[4];
-};
-__device__ __forceinline__ Coords site_coords(const LatGeo& g, int64_t s) {
-  Coords c;
-  uint32_t q = (uint32_t)s;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const uint32_t r = q / (uint32_t)g.L[d];
-    c.x[d] = (int32_t)(q - r * (uint32_t)g.L[d]);
-    q = r;
-  }
-  c.x[3] = (int32_t)q;
-  return c;
-}
-__device__ __forceinline__ int32_t neighbour(const LatGeo& g, const Coords& c, int32_t s, int mu,
-                                             bool bwd) {
-  const int32_t st = mu == 0 ? 1 : mu == 1 ? g.stride[1] : mu == 2 ? g.stride[2] : g.stride[3];
-  const int32_t L = mu == 0 ? g.L[0] : mu == 1 ? g.L[1] : mu == 2 ? g.L[2] : g.L[3];
-  const int32_t x = mu == 0 ? c.x[0] : mu == 1 ? c.x[1] : mu == 2 ? c.x[2] : c.x[3];
-  const int32_t wrap = (L - 1) * st;
-  return bwd ? (x == 0 ? s + wrap : s - st) : (x == L - 1 ? s - wrap : s + st);
-}
-
 // Direction of position t >> 1 in the order x, y, t, z.
 __device__ __forceinline__ int dir_at(int t) {
   const int p = t >> 1;

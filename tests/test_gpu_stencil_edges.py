@@ -71,3 +71,32 @@ def test_dslash_ragged_blocks_and_mixed_layouts(su3s, dims):
     su3s.dslash(z, U, P)
     ref = oracle.dslash(u, x.reshape(v, 4, 3, 2), dims).reshape(4 * v, 3, 2)
     assert np.abs(z.download() - ref).max() < 1.6e-12
+
+
+def test_vector_hop_with_special_inputs(su3s):
+    dims = (6, 5, 7, 9)
+    v = synth.volume(dims)
+    u, x = synth.su3(SEED, 4, 4 * v), synth.gauss_vector(SEED, 5, v)
+    plant(u, 40, 401)
+    plant(x, 333, 137)
+    lat = su3s.Lattice(dims)
+    U = field(su3s, lat, su3s.MATRIX, 4, u)
+    X = field(su3s, lat, su3s.VECTOR, 1, x)
+    z, zf = X.like(), X.like()
+    su3s.hop(z, U, X, su3s.MATH_DF32)
+    su3s.hop(zf, U, X, su3s.MATH_F64)
+    # 8 products of unit operands within 8e-13; operands up to 6 in size beside the planted ones
+    assert_like_native(z.download(), zf.download(), 8e-13 * 64)
+
+
+@pytest.mark.parametrize("dims", [(2, 1, 3, 43), (5, 51, 1, 1), (127, 1, 1, 1), (129, 2, 1, 1)])
+def test_vector_hop_ragged_blocks_and_mixed_layouts(su3s, dims):
+    v = synth.volume(dims)
+    u, x = synth.su3(SEED, 6, 4 * v), synth.gauss_vector(SEED, 7, v)
+    x /= np.abs(x).max()
+    lat = su3s.Lattice(dims)
+    U = field(su3s, lat, su3s.MATRIX, 4, u, su3s.AOSOA, 32)
+    X = field(su3s, lat, su3s.VECTOR, 1, x)
+    z = su3s.Field(lat, su3s.VECTOR, 1, su3s.F64, su3s.AOSOA, 4)
+    su3s.hop(z, U, X)
+    assert np.abs(z.download() - oracle.hop(u, x, dims)).max() < 8e-13
