@@ -395,6 +395,138 @@ __device__ __forceinline__ void df2_combine(DAcc2& a, const DAcc2& b) {
   a.lo = f2_add(a.lo, t);
 }
 
+// ------------------------------- MathDF, one operand of two values per lane pair
+// Where the two lanes hold operands of one shape each (the same real of two
+// sites, of two spins, of two products), the split FP64 inputs are the operands
+// as they stand: each lane performs MathDF's operations in MathDF's order.
+// dp: leading and trailing FP32 parts of one real of both; dpa: accumulator.
+using dp = df2;
+using dpa = DAcc2;
+
+__device__ __forceinline__ float2 f2_neg(float2 a) { return make_float2(-a.x, -a.y); }
+
+// a = +x*y (NEG: -x*y), MathDF::fma with FIRST.  With x negated every value of
+// the sequence is the exact negation of the positive one (round to nearest
+// even is symmetric), so the negative form negates the two results.  Zeros
+// are the exception (the leading product's +0 addend turns a -0 product into
+// +0): a result may differ from MathDF's in the sign of a zero, never in value.
+template <bool NEG>
+__device__ __forceinline__ void dp_first(dpa& a, const dp& x, const dp& y) {
+  const float2 p = f2_mul_lead(x.h, y.h);
+  const float2 np = f2_neg(p);
+  float2 q = f2_fma(x.h, y.h, np);  // exact error of the leading product
+  q = f2_fma(x.h, y.l, q);
+  q = f2_fma(x.l, y.h, q);
+  if (NEG) {
+    a.S = np;
+    a.lo = f2_neg(q);
+  } else {
+    a.S = p;
+    a.lo = q;
+  }
+}
+
+// a += x*y (NEG: a -= x*y), MathDF::fma without FIRST, lane-wise.  The
+// negative form is MathDF's sequence for -x written with x: s = S - p, the
+// error terms come out negated (c = -db, u = -t) and enter by subtraction
+// (equal values; the sign of a zero may differ, as in dp_first).
+template <bool NEG>
+__device__ __forceinline__ void dp_fma(dpa& a, const dp& x, const dp& y) {
+  const float2 p = f2_mul_lead(x.h, y.h);
+  if (!NEG) {
+    const float2 s = f2_add(a.S, p);        // TwoSum(S, xh*yh)
+    const float2 nbp = f2_sub(a.S, s);      // -bp
+    const float2 ap = f2_add(s, nbp);       // s - bp
+    const float2 db = f2_fma(x.h, y.h, nbp);
+    const float2 da = f2_sub(a.S, ap);
+    float2 t = f2_add(da, db);
+    t = f2_fma(x.l, y.h, t);
+    t = f2_fma(x.h, y.l, t);
+    a.S = s;
+    a.lo = f2_add(a.lo, t);
+  } else {
+    const float2 s = f2_sub(a.S, p);        // TwoSum(S, -xh*yh)
+    const float2 bp = f2_sub(s, a.S);
+    const float2 ap = f2_sub(s, bp);
+    const float2 c = f2_fma(x.h, y.h, bp);  // -db
+    const float2 da = f2_sub(a.S, ap);
+    float2 u = f2_sub(c, da);               // -(da + db)
+    u = f2_fma(x.l, y.h, u);
+    u = f2_fma(x.h, y.l, u);
+    a.S = s;
+    a.lo = f2_sub(a.lo, u);
+  }
+}
+
+// One complex term of SG * op(X) op(Y) into output (re, im): x = (xr, xm) and
+// y = (yr, ym) are the stored elements, op = adjoint when AX / AY.  The four
+// real terms enter in mm_acc's order: xr yr, xr ym, then xm ym, xm yr.
+template <bool FIRST, int SG, bool AX, bool AY>
+__device__ __forceinline__ void dp_cterm(dpa& re, dpa& im, const dp& xr, const dp& xm,
+                                         const dp& yr, const dp& ym) {
+  constexpr int sx = AX ? -1 : 1, sy = AY ? -1 : 1;
+  if constexpr (FIRST) {
+    dp_first<(SG < 0)>(re, xr, yr);
+    dp_first<(SG * sy < 0)>(im, xr, ym);
+  } else {
+    dp_fma<(SG < 0)>(re, xr, yr);
+    dp_fma<(SG * sy < 0)>(im, xr, ym);
+  }
+  dp_fma<(-SG * sx * sy < 0)>(re, xm, ym);
+  dp_fma<(SG * sx < 0)>(im, xm, yr);
+}
+
+// N independent terms a[n] += x * y[n] (bit n of NEG: a[n] -= x * y[n]) that
+// share the operand x, step by step side by side: the operations of dp_fma
+// (FIRST: dp_first) in its order for each, so that consecutive FMAs read x's
+// register pair once.  The register file feeds two 32-bit operands per cycle
+// and scheduler: a packed FMA of three different pairs takes 3 cycles, with one
+// of them held over from the instruction before 2.2 (measured, 1 to 4 warps per
+// scheduler; packed additions 2.0), so the products are bound by operand reads
+// unless they share them.
+template <int N, bool FIRST, uint32_t NEG>
+__device__ __forceinline__ void dp_fma_shared(dpa* const (&a)[N], const dp& x, const dp* const (&y)[N]) {
+  float2 p[N], s[N], b[N], c[N], t[N];
+#pragma unroll
+  for (int n = 0; n < N; ++n) p[n] = f2_mul_lead(x.h, y[n]->h);
+  if constexpr (FIRST) {
+#pragma unroll
+    for (int n = 0; n < N; ++n) t[n] = f2_fma(x.h, y[n]->h, f2_neg(p[n]));
+#pragma unroll
+    for (int n = 0; n < N; ++n) t[n] = f2_fma(x.h, y[n]->l, t[n]);
+#pragma unroll
+    for (int n = 0; n < N; ++n) t[n] = f2_fma(x.l, y[n]->h, t[n]);
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+      const bool neg = (NEG >> n) & 1u;
+      a[n]->S = neg ? f2_neg(p[n]) : p[n];
+      a[n]->lo = neg ? f2_neg(t[n]) : t[n];
+    }
+  } else {
+#pragma unroll
+    for (int n = 0; n < N; ++n) s[n] = (NEG >> n) & 1u ? f2_sub(a[n]->S, p[n]) : f2_add(a[n]->S, p[n]);
+#pragma unroll
+    for (int n = 0; n < N; ++n) b[n] = (NEG >> n) & 1u ? f2_sub(s[n], a[n]->S) : f2_sub(a[n]->S, s[n]);
+#pragma unroll
+    for (int n = 0; n < N; ++n) c[n] = (NEG >> n) & 1u ? f2_sub(s[n], b[n]) : f2_add(s[n], b[n]);  // s - bp
+#pragma unroll
+    for (int n = 0; n < N; ++n) b[n] = f2_fma(x.h, y[n]->h, b[n]);   // +-db
+#pragma unroll
+    for (int n = 0; n < N; ++n) c[n] = f2_sub(a[n]->S, c[n]);        // da
+#pragma unroll
+    for (int n = 0; n < N; ++n) t[n] = (NEG >> n) & 1u ? f2_sub(b[n], c[n]) : f2_add(c[n], b[n]);
+#pragma unroll
+    for (int n = 0; n < N; ++n) t[n] = f2_fma(x.l, y[n]->h, t[n]);
+#pragma unroll
+    for (int n = 0; n < N; ++n) t[n] = f2_fma(x.h, y[n]->l, t[n]);
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+      a[n]->S = s[n];
+      a[n]->lo = (NEG >> n) & 1u ? f2_sub(a[n]->lo, t[n]) : f2_add(a[n]->lo, t[n]);
+    }
+  }
+}
+
 // -------------------------------------------------------------- MathFX
 // One real of an object: value (h * 2^25 + l * 2^-6) * 2^(e - 1075), with
 // |h| <= 2^28, |l| < 2^31 and l a multiple of 64 (the low 25 bits of m,

@@ -25,11 +25,6 @@
 
 namespace su3s {
 
-// one real of the two sites: leading and trailing FP32 parts, lane k = site k
-using dp = df2;
-// accumulator of one real of the two sites (MathDF's DAcc, lane-wise)
-using dpa = DAcc2;
-
 // df_split_bits of two FP64 values (the same real of the two sites).
 __device__ __forceinline__ dp dp_split(uint32_t lo0, uint32_t hi0, uint32_t lo1, uint32_t hi1) {
   return df2_split(lo0, hi0, lo1, hi1);
@@ -38,79 +33,6 @@ __device__ __forceinline__ dp dp_split(uint32_t lo0, uint32_t hi0, uint32_t lo1,
 // df_to_double of both lanes.
 __device__ __forceinline__ void dp_to_double(const dpa& a, double& d0, double& d1) {
   df2_to_double(a, d0, d1);
-}
-
-__device__ __forceinline__ float2 f2_neg(float2 a) { return make_float2(-a.x, -a.y); }
-
-// a = +x*y (NEG: -x*y), MathDF::fma with FIRST.  With x negated every value of
-// the sequence is the exact negation of the positive one (round to nearest
-// even is symmetric), so the negative form negates the two results.  Zeros
-// are the exception (the leading product's +0 addend turns a -0 product into
-// +0): a result may differ from MathDF's in the sign of a zero, never in value.
-template <bool NEG>
-__device__ __forceinline__ void dp_first(dpa& a, const dp& x, const dp& y) {
-  const float2 p = f2_mul_lead(x.h, y.h);
-  const float2 np = f2_neg(p);
-  float2 q = f2_fma(x.h, y.h, np);  // exact error of the leading product
-  q = f2_fma(x.h, y.l, q);
-  q = f2_fma(x.l, y.h, q);
-  if (NEG) {
-    a.S = np;
-    a.lo = f2_neg(q);
-  } else {
-    a.S = p;
-    a.lo = q;
-  }
-}
-
-// a += x*y (NEG: a -= x*y), MathDF::fma without FIRST, lane-wise.  The
-// negative form is MathDF's sequence for -x written with x: s = S - p, the
-// error terms come out negated (c = -db, u = -t) and enter by subtraction
-// (equal values; the sign of a zero may differ, as in dp_first).
-template <bool NEG>
-__device__ __forceinline__ void dp_fma(dpa& a, const dp& x, const dp& y) {
-  const float2 p = f2_mul_lead(x.h, y.h);
-  if (!NEG) {
-    const float2 s = f2_add(a.S, p);        // TwoSum(S, xh*yh)
-    const float2 nbp = f2_sub(a.S, s);      // -bp
-    const float2 ap = f2_add(s, nbp);       // s - bp
-    const float2 db = f2_fma(x.h, y.h, nbp);
-    const float2 da = f2_sub(a.S, ap);
-    float2 t = f2_add(da, db);
-    t = f2_fma(x.l, y.h, t);
-    t = f2_fma(x.h, y.l, t);
-    a.S = s;
-    a.lo = f2_add(a.lo, t);
-  } else {
-    const float2 s = f2_sub(a.S, p);        // TwoSum(S, -xh*yh)
-    const float2 bp = f2_sub(s, a.S);
-    const float2 ap = f2_sub(s, bp);
-    const float2 c = f2_fma(x.h, y.h, bp);  // -db
-    const float2 da = f2_sub(a.S, ap);
-    float2 u = f2_sub(c, da);               // -(da + db)
-    u = f2_fma(x.l, y.h, u);
-    u = f2_fma(x.h, y.l, u);
-    a.S = s;
-    a.lo = f2_sub(a.lo, u);
-  }
-}
-
-// One complex term of SG * op(X) op(Y) into output (re, im): x = (xr, xm) and
-// y = (yr, ym) are the stored elements, op = adjoint when AX / AY.  The four
-// real terms enter in mm_acc's order: xr yr, xr ym, then xm ym, xm yr.
-template <bool FIRST, int SG, bool AX, bool AY>
-__device__ __forceinline__ void dp_cterm(dpa& re, dpa& im, const dp& xr, const dp& xm,
-                                         const dp& yr, const dp& ym) {
-  constexpr int sx = AX ? -1 : 1, sy = AY ? -1 : 1;
-  if constexpr (FIRST) {
-    dp_first<(SG < 0)>(re, xr, yr);
-    dp_first<(SG * sy < 0)>(im, xr, ym);
-  } else {
-    dp_fma<(SG < 0)>(re, xr, yr);
-    dp_fma<(SG * sy < 0)>(im, xr, ym);
-  }
-  dp_fma<(-SG * sx * sy < 0)>(re, xm, ym);
-  dp_fma<(SG * sx < 0)>(im, xm, yr);
 }
 
 // ------------------------------------------------------- operand sources

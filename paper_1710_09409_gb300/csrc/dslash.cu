@@ -342,7 +342,8 @@ __global__ void __launch_bounds__(kDslashThreads) k_dslash(FieldDesc dst, FieldD
 // Measured at 32^3 x 64 (pair arithmetic, default launch): 1,031 us before (one
 // (re, im) pair per lane pair, 242 registers, 10,870 instructions per site),
 // 884 us with the spins packed, 787 with the colours pipelined (8,580
-// instructions), 755 with four waves of blocks, 740 with walked addresses.
+// instructions), 755 with four waves of blocks, 740 with walked addresses, 728
+// with the six terms of a colour side by side (dp_fma_shared).
 // Not kept: tiles of sites in 2, 3 or 4 dimensions per block with and without
 // L1 (863-880 against 873 us), 128 registers (815), the first term opening the
 // accumulators (761 against 755).
@@ -530,15 +531,22 @@ __global__ void __launch_bounds__(kDslashThreads, 3)
         const TermForm& fr = j < 2 ? fc : fn;
         uint32_t& gr = j < 2 ? gm : gm_next;
         read_half(nxt, slot, fr, jn, gr);
+        dp er[3], em[3];
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
           const df2& e = cur.u[i];
-          const dp er{make_float2(e.h.x, e.h.x), make_float2(e.l.x, e.l.x)};
-          const dp em{make_float2(e.h.y, e.h.y), make_float2(e.l.y, e.l.y)};
-          if (j == 0) dp_cterm<true, 1, false, false>(re[i], im[i], er, em, cur.hr, cur.hm);
-          else dp_cterm<false, 1, false, false>(re[i], im[i], er, em, cur.hr, cur.hm);
-          read_link_elem(nxt, slot, fr, jn, i, gr);
+          er[i] = dp{make_float2(e.h.x, e.h.x), make_float2(e.l.x, e.l.x)};
+          em[i] = dp{make_float2(e.h.y, e.h.y), make_float2(e.l.y, e.l.y)};
         }
+        dpa* const a0[6] = {&re[0], &re[1], &re[2], &im[0], &im[1], &im[2]};
+        const dp* const y0[6] = {&er[0], &er[1], &er[2], &em[0], &em[1], &em[2]};
+        const dp* const y1[6] = {&em[0], &em[1], &em[2], &er[0], &er[1], &er[2]};
+        if (j == 0) dp_fma_shared<6, true, 0u>(a0, cur.hr, y0);
+        else dp_fma_shared<6, false, 0u>(a0, cur.hr, y0);
+        read_link_elem(nxt, slot, fr, jn, 0, gr);
+        read_link_elem(nxt, slot, fr, jn, 1, gr);
+        dp_fma_shared<6, false, 7u>(a0, cur.hm, y1);
+        read_link_elem(nxt, slot, fr, jn, 2, gr);
         cur = nxt;
       }
       const float2 f = make_float2(__uint_as_float((fc.i0 & 0x80000000u) | 0x3F800000u),
