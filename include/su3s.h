@@ -349,8 +349,8 @@ int su3s_device_error(int* code, void* stream);
 int su3s_selftest_bounded_wait(uint32_t polls, int64_t* cycles, void* stream);
 
 /* Autotune the launch geometry for `e` into `dest`: times each candidate
- * (data movement 0..4 as for su3s_set_pipeline, threads 64..256, full or
- * grid-stride grids) with CUDA events on `stream` (synchronising it; dest is
+ * (data movement 0..4 as for su3s_set_pipeline, threads 64..256, or 512 for
+ * trees whose default that is, full or grid-stride grids) with CUDA events on `stream` (synchronising it; dest is
  * overwritten, so a dest that is one of the leaves changes that leaf), keeps
  * the fastest for later su3s_eval calls and reports it in
  * *threads, *blocks_per_sm, *variant and its time in *best_ms (any may be

@@ -183,7 +183,7 @@ static int staged_occupancy(const void* kernel, int threads, int warp_bytes) {
   int n = 0;
   const size_t smem = (size_t)(threads / 32) * warp_bytes;
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       8 * warp_bytes < smem_optin() ? 8 * warp_bytes : smem_optin());
+                       staged_smem_max(warp_bytes));
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess || n < 1)
     n = 1;
   cache[key] = n;
@@ -215,13 +215,15 @@ int plan_launch(const EvalEntry* e, int64_t nvec, int nmu, bool tma_ok, Launch* 
   }
   if (variant > 0) {
     int threads = g.threads > 0 ? g.threads : 128;
+    if (threads > 256 && variant != e->default_variant) threads = 256;
     if ((variant == 2 || variant == 3) && threads > 128) threads = 128;  // per-leaf / ring: <= 4 warps
     // at most the warps whose buffers fit one block's shared memory
-    while (threads > 32 && (threads / 32) * e->warp_bytes[variant] > smem_optin()) threads -= 32;
+    while (threads > 32 && (threads / 32) * e->warp_bytes[variant] > staged_smem_limit()) threads -= 32;
+    // warps take 32-site tiles, or units of two tiles (two sites per lane)
+    const int64_t ntiles = variant == 4 ? (nvec / 32 + 1) / 2 : nvec / 32;
     const int occ = staged_occupancy(e->kernel[variant], threads, e->warp_bytes[variant]);
     const int per_sm = g.bps > 0 && g.bps < occ ? g.bps : occ;
-    // warps take 32-site tiles, or units of two tiles (two sites per lane)
-    const int64_t ntiles = variant == 4 ? (nvec / 32 + 1) / 2 : nvec / 32, wpb = threads / 32;
+    const int64_t wpb = threads / 32;
     int64_t nb = ((int64_t)per_sm * sm_count() + nmu - 1) / nmu;
     const int64_t need = (ntiles + wpb - 1) / wpb;
     if (nb > need) nb = need;
@@ -248,7 +250,7 @@ void launch_geometry(const void* kernel, int64_t nvec, int nmu, dim3* grid, dim3
 // grid of bps blocks per SM, else one site vector per thread.
 void plain_geometry(int threads, int bps, int64_t nvec, int nmu, dim3* grid, dim3* block) {
   Geo g{threads, bps, -1};
-  if (g.threads <= 0) g.threads = 256;
+  if (g.threads <= 0 || g.threads > 256) g.threads = 256;
   int64_t nb;
   if (g.bps > 0) {
     nb = (int64_t)g.bps * sm_count();
@@ -913,7 +915,7 @@ static int tune_entry(const EvalEntry* ent, const void* params, int64_t nvec, in
     cudaEventDestroy(e0);
     return fail(SU3S_ECUDA, "event creation failed");
   }
-  const int th_c[] = {64, 128, 256};
+  const int th_c[] = {64, 128, 256, 512};
   const int bps_c[] = {0, 2, 4, 8};
   const bool tma = ent->fn[1] && tma_ok && nvec % 32 == 0;
   float best = 1e30f;
@@ -923,6 +925,8 @@ static int tune_entry(const EvalEntry* ent, const void* params, int64_t nvec, in
     if (!ent->fn[var]) continue;
     for (int th : th_c) {
       if ((var == 2 || var == 3) && th > 128) continue;  // per-leaf / ring: at most 4 warps
+      // one block of 16 warps: only the kernels whose default it is take it
+      if (th > 256 && (var != ent->default_variant || ent->default_threads != th)) continue;
       for (int bps : bps_c) {
         set_geometry(ent->kernel[0], nvec, nmu, th, bps, var);
         Launch L;

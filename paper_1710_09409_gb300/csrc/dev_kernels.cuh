@@ -280,6 +280,45 @@ __device__ __forceinline__ Range warp_range(int64_t end) {
   return Range{(int64_t)blockIdx.x * nw + (threadIdx.x >> 5), end, (int64_t)gridDim.x * nw};
 }
 
+// A warp's units in the order of warp_range: a fixed share, one unit every
+// grid's worth of warps.
+struct UnitStride {
+  int64_t end, t;
+  __device__ __forceinline__ int64_t open() {
+    const Range r = warp_range(end);
+    t = r.first;
+    return t;
+  }
+  __device__ __forceinline__ int64_t next(int) {
+    t += (int64_t)gridDim.x * (blockDim.x >> 5);
+    return t;
+  }
+};
+// The same units handed out as the block's warps come.  For kernels that run
+// one block of many warps per SM and are bound by issue or register reads: the
+// schedulers then do not serve the warps evenly, and with fixed shares those
+// served first leave the others alone at the end (see CommutatorOk).
+struct UnitQueue {
+  int64_t end;
+  int* taken;   // shared memory: units of the block handed out so far
+  // Every thread of the block calls it (it synchronises); returns the warp's
+  // first unit.
+  __device__ __forceinline__ int64_t open() {
+    if (threadIdx.x == 0) *taken = blockDim.x >> 5;
+    __syncthreads();
+    return (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  }
+  // The warp's next unit (>= end: none left).
+  __device__ __forceinline__ int64_t next(int lane) {
+    const uint32_t nw = blockDim.x >> 5;
+    uint32_t k = 0;
+    if (lane == 0) k = (uint32_t)atomicAdd(taken, 1);
+    k = __shfl_sync(0xffffffffu, k, 0);
+    const uint32_t r = k / nw;
+    return ((int64_t)r * gridDim.x + blockIdx.x) * nw + (k - r * nw);
+  }
+};
+
 template <class Tree, class M, int PREC>
 __device__ __forceinline__ void plain_range(const KParams& p, Range r) {
   const int mu = blockIdx.y;
@@ -523,17 +562,29 @@ struct TwoProducts<Add<X, Y>> : TwoProductsOf<X, Y, 1> {};
 template <class X, class Y>
 struct TwoProducts<Sub<X, Y>> : TwoProductsOf<X, Y, -1> {};
 
-// Sums and differences of two 3x3 products whose leaves overlap
-// (adj(a)*b - b*adj(a)): every leaf stays live through both products, so the
-// whole-tile kernel evaluates the output one row at a time -- the first
-// product's row into three accumulators, the second's row combined into them,
-// the row converted and stored -- and holds three outputs' accumulators
-// instead of the eighteen of both products.  Each output's operations are
-// acc_node's and mul_combine's in the same order: the values are unchanged.
-// Pair arithmetic with packed (re, im) lanes, full FP64 matrices.
+// Commutators and anticommutators x y -+ y x of two matrix leaves or adjoints
+// (adj(a)*b - b*adj(a)): the two products read the same operands, so the
+// whole-tile kernel puts one in each lane of the packed FP32 operations, xy in
+// lane 0 and yx in lane 1.  An element pair (x_ij, y_ij) is what the left
+// factors need and its lanes swapped are the right ones: nothing is duplicated
+// or signed (an adjoint is a transposed read and a sign folded into the split),
+// where (re, im) packing builds signed and swapped copies of both operands for
+// both products.  The output goes row by row: both products' row, the lanes
+// combined, the row stored.  Each output's operations are acc_node's and
+// mul_combine's in the same order: the values are those of the other data
+// movements.  Pair arithmetic, full FP64 matrices.
+// Bound by register reads: 3,440 scheduler cycles per tile at 40^4 against
+// about 3,300 of operand reads (see dp_fma_shared).  Measured at 40^4: 243 us
+// with (re, im) lanes (2,190 instructions per site, two blocks of 8 warps per
+// SM), 225 with the products in the lanes (1,900), 222 with one block of 16
+// warps and a queue of tiles (of the two blocks one had run ahead and ended at
+// 138 us, leaving the SM half empty), 219 with the terms side by side
+// (dp_fma_shared).  12 warps of 164 registers 226, 8 of 252 226.
 template <class T>
 struct MatLeafOperand {
   static constexpr bool value = false;
+  static constexpr int slot = -1;
+  static constexpr bool adj = false;
 };
 template <int J>
 struct MatLeafOperand<LM<J>> {
@@ -545,59 +596,90 @@ struct MatLeafOperand<Adj<LM<J>>> {
   static constexpr bool value = true, adj = true;
   static constexpr int slot = J;
 };
+template <class A, class B>
+constexpr bool same_operand() {
+  using X = MatLeafOperand<A>;
+  using Y = MatLeafOperand<B>;
+  return X::value && Y::value && X::slot == Y::slot && X::adj == Y::adj;
+}
 template <class T>
-struct MatLeafProduct {
+struct Commutator {
   static constexpr bool value = false;
 };
-template <class X, class Y>
-struct MatLeafProduct<Mul<X, Y>> {
-  using LX = MatLeafOperand<X>;
-  using LY = MatLeafOperand<Y>;
-  static constexpr bool value = LX::value && LY::value;
-};
-template <class T>
-struct RowProducts {
-  static constexpr bool value = false;
-};
-template <class X, class Y, int SG>
-struct RowProductsOf {
-  static constexpr bool value =
-      MatLeafProduct<X>::value && MatLeafProduct<Y>::value && !disjoint_leaves<X, Y, 0>();
-  using P0 = MatLeafProduct<X>;
-  using P1 = MatLeafProduct<Y>;
+template <class X0, class Y0, class X1, class Y1, int SG>
+struct CommutatorOf {
+  static constexpr bool value = same_operand<X0, Y1>() && same_operand<Y0, X1>();
+  using X = MatLeafOperand<X0>;
+  using Y = MatLeafOperand<Y0>;
   static constexpr int S1 = SG;
 };
-template <class X, class Y>
-struct RowProducts<Add<X, Y>> : RowProductsOf<X, Y, 1> {};
-template <class X, class Y>
-struct RowProducts<Sub<X, Y>> : RowProductsOf<X, Y, -1> {};
+template <class X0, class Y0, class X1, class Y1>
+struct Commutator<Add<Mul<X0, Y0>, Mul<X1, Y1>>> : CommutatorOf<X0, Y0, X1, Y1, 1> {};
+template <class X0, class Y0, class X1, class Y1>
+struct Commutator<Sub<Mul<X0, Y0>, Mul<X1, Y1>>> : CommutatorOf<X0, Y0, X1, Y1, -1> {};
 
 template <class Tree, class M, int PREC>
-struct RowProductsOk {
-  static constexpr bool value = RowProducts<Tree>::value && M::kPaired && PREC == P_F64;
+struct CommutatorOk {
+  static constexpr bool value = Commutator<Tree>::value && M::kPaired && PREC == P_F64;
 };
 
-// Evaluate and store site s, row by row (RowProductsOk holds).
-template <class Tree, class M, class C>
-__device__ __forceinline__ void row_products_store(const FieldDesc& f, const C& ctx, int64_t s,
-                                                   int mu) {
-  using RP = RowProducts<Tree>;
-  using X0 = typename RP::P0::LX;
-  using Y0 = typename RP::P0::LY;
-  using X1 = typename RP::P1::LX;
-  using Y1 = typename RP::P1::LY;
+// w[2 (3 i + j)], w[2 (3 i + j) + 1]: real and imaginary part of (x_ij, y_ij)
+// of this lane's site, from the staged tile.
+template <class Tree, int PREC>
+__device__ __forceinline__ void read_commutator(const unsigned char* buf, int lane, df2* w,
+                                                uint32_t& gm) {
+  using C = Commutator<Tree>;
+  using X = typename C::X;
+  using Y = typename C::Y;
+  const uint4* px = reinterpret_cast<const uint4*>(buf + LeafOff<Tree, PREC, X::slot>::value) + lane;
+  const uint4* py = reinterpret_cast<const uint4*>(buf + LeafOff<Tree, PREC, Y::slot>::value) + lane;
+  constexpr uint32_t nx = X::adj ? 0x80000000u : 0u, ny = Y::adj ? 0x80000000u : 0u;
+  uint32_t g[9];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int e = 3 * i + j, t = 3 * j + i;
+      const uint4 a = px[(X::adj ? t : e) * 32], b = py[(Y::adj ? t : e) * 32];
+      g[e] = guard_max(guard_max(0u, a.y, a.w), b.y, b.w);
+      w[2 * e] = df2_split(a.x, a.y, b.x, b.y);
+      w[2 * e + 1] = df2_split(a.z, a.w ^ nx, b.z, b.w ^ ny);
+    }
+  gm = max(gm, guard_reduce<9>(g));
+}
+
+__device__ __forceinline__ df2 df2_swap(const df2& a) {
+  return df2{make_float2(a.h.y, a.h.x), make_float2(a.l.y, a.l.x)};
+}
+
+// Evaluate and store site s, row by row (CommutatorOk holds).
+template <class Tree>
+__device__ __forceinline__ void commutator_store(const FieldDesc& f, const df2* w, int64_t s, int mu) {
   const int64_t b = elem_base(f, s, mu);
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    DAcc2 P[3], Q[3];
-    mm_pairs_row2<X0::adj, Y0::adj, X1::adj, Y1::adj>(P, Q, ctx.leaf[X0::slot], ctx.leaf[Y0::slot],
-                                                      ctx.leaf[X1::slot], ctx.leaf[Y1::slot], i);
+    dpa re[3], im[3];   // lanes: (xy)_ik, (yx)_ik
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const dp xr = w[2 * (3 * i + j)], xm = w[2 * (3 * i + j) + 1];
+      dp y[6];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) y[k] = df2_swap(w[6 * j + k]);
+      dpa* const a0[6] = {&re[0], &re[1], &re[2], &im[0], &im[1], &im[2]};
+      const dp* const y0[6] = {&y[0], &y[2], &y[4], &y[1], &y[3], &y[5]};
+      const dp* const y1[6] = {&y[1], &y[3], &y[5], &y[0], &y[2], &y[4]};
+      if (j == 0) dp_fma_shared<6, true, 0u>(a0, xr, y0);
+      else dp_fma_shared<6, false, 0u>(a0, xr, y0);
+      dp_fma_shared<6, false, 7u>(a0, xm, y1);
+    }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      df2_combine<RP::S1>(P[k], Q[k]);
-      typename M::A re, im;
-      dacc2_put(re, im, P[k]);
-      Store<P_F64>::template store_acc<M>(f.ptr, b + (3 * i + k) * f.s_c, &re, &im);
+      DAcc2 z{make_float2(re[k].S.x, im[k].S.x), make_float2(re[k].lo.x, im[k].lo.x)};
+      const DAcc2 q{make_float2(re[k].S.y, im[k].S.y), make_float2(re[k].lo.y, im[k].lo.y)};
+      df2_combine<Commutator<Tree>::S1>(z, q);
+      DAcc zr, zm;
+      dacc2_put(zr, zm, z);
+      Store<P_F64>::template store_acc<MathDF>(f.ptr, b + (3 * i + k) * f.s_c, &zr, &zm);
     }
   }
 }
@@ -612,8 +694,8 @@ __device__ __forceinline__ void read_leaves_of(const unsigned char* buf, int lan
   }
 }
 
-template <class Tree, class M, int PREC>
-__device__ __forceinline__ void tma_range(const KParams& p, Range rg, unsigned char* smem) {
+template <class Tree, class M, int PREC, class Units>
+__device__ __forceinline__ void tma_range(const KParams& p, Units q, unsigned char* smem) {
   constexpr int NL = Tree::nleaf;
   constexpr int NS = Tree::nsc;
   constexpr int W = Width<Tree::kind>::value;
@@ -622,9 +704,8 @@ __device__ __forceinline__ void tma_range(const KParams& p, Range rg, unsigned c
   unsigned char* buf = smem + warp * tma_warp_stride(TB);
   uint64_t* bar = reinterpret_cast<uint64_t*>(buf + TB);
   const int mu = blockIdx.y;
-  const int64_t ntiles = rg.end;
-  const int64_t wstride = rg.stride;
-  int64_t t = rg.first;
+  const int64_t ntiles = q.end;
+  int64_t t = q.open();
   if (lane == 0) {
     mbar_init(bar, 1);
     fence_barrier_init();
@@ -643,16 +724,17 @@ __device__ __forceinline__ void tma_range(const KParams& p, Range rg, unsigned c
     }
     phase ^= 1;
     ctx.gmax = p.gscal;
-    const int64_t tn = t + wstride;
-    if constexpr (RowProductsOk<Tree, M, PREC>::value) {
-      read_leaves<Tree, 0, PREC, M>(buf, lane, ctx);
+    const int64_t tn = q.next(lane);
+    if constexpr (CommutatorOk<Tree, M, PREC>::value) {
+      df2 w[18];
+      read_commutator<Tree, PREC>(buf, lane, w, ctx.gmax);
       fence_proxy_async_smem();
       __syncwarp();
       if (tn < ntiles) issue_tile<Tree, PREC, false>(lane, p, nullptr, nullptr, tn << 5, mu, buf, bar);
       if (M::kGuard && __any_sync(0xffffffffu, guard_trips<Tree>(ctx.gmax)))
         eval_site_f64<Tree, PREC>(p, (t << 5) + lane, mu);
       else
-        row_products_store<Tree, M>(p.dst, ctx, (t << 5) + lane, mu);
+        commutator_store<Tree>(p.dst, w, (t << 5) + lane, mu);
       t = tn;
       continue;
     }
@@ -700,25 +782,33 @@ __device__ __forceinline__ void tma_range(const KParams& p, Range rg, unsigned c
 }
 
 // Minimum blocks per SM the whole-tile kernel declares, which steers the
-// registers ptxas gives it: row-by-row products fit 128 registers (two blocks
-// of 256 threads); the other full-matrix trees in the pair arithmetic are given
+// registers ptxas gives it: full-matrix trees in the pair arithmetic are given
 // the registers of one block (more independent work per warp: a*b+c*d 234
 // instead of 186 registers at the same 8 warps per SM, and measured faster);
 // two-row matrices and the other arithmetics state no minimum (two-row a*b: 107
 // registers and many warps, 10% faster than with one block's 148).
 template <class Tree, class M, int PREC>
 struct TmaMinBlocks {
-  static constexpr int value = RowProductsOk<Tree, M, PREC>::value        ? 2
-                               : (PREC == P_F64 && M::kPaired) ? 1
-                                                                : 0;
+  static constexpr int value = PREC == P_F64 && M::kPaired ? 1 : 0;
+};
+// Most threads of a whole-tile launch: commutators run as one block of 16 warps
+// per SM (128 registers).
+template <class Tree, class M, int PREC>
+struct TmaMaxThreads {
+  static constexpr int value = CommutatorOk<Tree, M, PREC>::value ? 512 : 256;
 };
 
 template <class Tree, class M, int PREC>
-__global__ void __launch_bounds__(256, TmaMinBlocks<Tree, M, PREC>::value)
+__global__ void __launch_bounds__(TmaMaxThreads<Tree, M, PREC>::value, TmaMinBlocks<Tree, M, PREC>::value)
     k_eval_tma(const __grid_constant__ KParams p) {
   extern __shared__ __align__(128) unsigned char smem[];
   if (!smem_aligned(smem, p.err)) return;
-  tma_range<Tree, M, PREC>(p, warp_range(p.nvec >> 5), smem);
+  if constexpr (CommutatorOk<Tree, M, PREC>::value) {
+    __shared__ int taken;
+    tma_range<Tree, M, PREC>(p, UnitQueue{p.nvec >> 5, &taken}, smem);
+  } else {
+    tma_range<Tree, M, PREC>(p, UnitStride{p.nvec >> 5, 0}, smem);
+  }
 }
 
 template <class Tree, class M>
@@ -1403,6 +1493,13 @@ inline int smem_optin() {
   return v;
 }
 
+// Dynamic shared memory a staged block can have (its unit counter is static),
+// and the most a staged launch may ask for: 16 warps' buffers, as far as they fit.
+inline int staged_smem_limit() { return smem_optin() - 1024; }
+inline int staged_smem_max(int warp_bytes) {
+  return 16 * warp_bytes < staged_smem_limit() ? 16 * warp_bytes : staged_smem_limit();
+}
+
 // Dynamic shared memory of a TMA-staged launch: one tile buffer and one
 // barrier per warp.
 inline size_t tma_smem(int tile_bytes, dim3 block) {
@@ -1417,7 +1514,7 @@ cudaError_t launch_eval_tma(const void* params, dim3 grid, dim3 block, cudaStrea
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(k_eval_tma<Tree, M, PREC>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         8 * tma_warp_stride(TB));
+                                         staged_smem_max(tma_warp_stride(TB)));
     if (e != cudaSuccess) return e;
     attr = true;
   }
@@ -1433,7 +1530,7 @@ cudaError_t launch_adjoint_tma(const void* params, dim3 grid, dim3 block, cudaSt
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(k_adjoint_tma<Tree, M>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         8 * tma_warp_stride(TB));
+                                         staged_smem_max(tma_warp_stride(TB)));
     if (e != cudaSuccess) return e;
     attr = true;
   }
@@ -1447,7 +1544,7 @@ cudaError_t launch_eval_lazy(const void* params, dim3 grid, dim3 block, cudaStre
   static bool attr = false;
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(k_eval_lazy<Tree, M, PREC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * S);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, staged_smem_max(S));
     if (e != cudaSuccess) return e;
     attr = true;
   }
@@ -1461,7 +1558,7 @@ cudaError_t launch_adjoint_lazy(const void* params, dim3 grid, dim3 block, cudaS
   static bool attr = false;
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(k_adjoint_lazy<Tree, M>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * S);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, staged_smem_max(S));
     if (e != cudaSuccess) return e;
     attr = true;
   }
@@ -1475,7 +1572,7 @@ cudaError_t launch_eval_ring(const void* params, dim3 grid, dim3 block, cudaStre
   static bool attr = false;
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(k_eval_ring<Tree, M, PREC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * S);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, staged_smem_max(S));
     if (e != cudaSuccess) return e;
     attr = true;
   }
@@ -1489,7 +1586,7 @@ cudaError_t launch_adjoint_ring(const void* params, dim3 grid, dim3 block, cudaS
   static bool attr = false;
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(k_adjoint_ring<Tree, M>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * S);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, staged_smem_max(S));
     if (e != cudaSuccess) return e;
     attr = true;
   }
@@ -1582,6 +1679,7 @@ constexpr DefaultGeo default_geometry() {
   // in small blocks, about 8 warps per SM (16 for matrix times vector); the
   // rest with the most that fit.
   if constexpr (M::kScaled) return DefaultGeo{1, 128, 0};
+  else if constexpr (!GRAD && CommutatorOk<Tree, M, PREC>::value) return DefaultGeo{1, 512, 1};
   else if constexpr (GRAD && pair_adjoint_ok<Tree, M>()) return DefaultGeo{4, 256, 0};
   else if constexpr (!GRAD && PREC == P_F64 && IsLeafProduct<Tree>::value)
     return Tree::kind == KV ? DefaultGeo{1, 64, 8} : DefaultGeo{1, 64, 4};
@@ -1595,7 +1693,7 @@ cudaError_t launch_eval_pair(const void* params, dim3 grid, dim3 block, cudaStre
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(k_eval_pair<Tree>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         8 * S < smem_optin() ? 8 * S : smem_optin());
+                                         staged_smem_max(S));
     if (e != cudaSuccess) return e;
     attr = true;
   }
@@ -1610,7 +1708,7 @@ cudaError_t launch_adjoint_pair(const void* params, dim3 grid, dim3 block, cudaS
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(k_adjoint_pair<Tree>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         8 * S < smem_optin() ? 8 * S : smem_optin());
+                                         staged_smem_max(S));
     if (e != cudaSuccess) return e;
     attr = true;
   }
