@@ -221,6 +221,30 @@ int plan_launch(const EvalEntry* e, int64_t nvec, int nmu, bool tma_ok, Launch* 
     while (threads > 32 && (threads / 32) * e->warp_bytes[variant] > staged_smem_limit()) threads -= 32;
     // warps take 32-site tiles, or units of two tiles (two sites per lane)
     const int64_t ntiles = variant == 4 ? (nvec / 32 + 1) / 2 : nvec / 32;
+    // one block of 16 warps per SM pays from about 96 tiles per SM on (its warps
+    // take tiles from one queue, so they end together, but also begin their
+    // last, incomplete round together); below, four blocks of 4 warps:
+    // adj(a)*b - b*adj(a) 17^4 10.6 against 15.9 us, 24^4 35.4 / 39.4, 26^4
+    // 46.5 / 46.6, 28^4 60.3 / 59.1, 40^4 228 / 217
+    if (!set && threads > 256 && ntiles * nmu < (int64_t)96 * sm_count()) {
+      threads = 128;
+      g.bps = 4;
+    }
+    // likewise one block of 8 warps per SM below 40 tiles per SM: the tiles left
+    // over from whole rounds then go to warps of more SMs (a*b + c*d 17^4 14.2 ->
+    // 12.0 us, 20^4 23.0 -> 21.8, 22^4 33.5 either way; 0.5 a + b 20^4 8.8 -> 8.2)
+    else if (!set && threads == 256 && g.bps == 0 && ntiles * nmu < (int64_t)40 * sm_count()) {
+      threads = 128;
+    }
+    // small lattices, default launch: smaller blocks (and as many more per SM)
+    // until every SM has one.  A single tile's time is its instructions'
+    // latency, so tiles spread over the SMs: 8^4 a*b + c*d 6.0 -> 4.8 us,
+    // (a*b)*c + 0.5*d 6.3 -> 5.1, adj(a)*b - b*adj(a) 5.5 -> 3.6.
+    if (!set)
+      while (threads > 32 && threads % 64 == 0 && ntiles * nmu < (int64_t)(threads / 32) * sm_count()) {
+        threads /= 2;
+        g.bps *= 2;
+      }
     const int occ = staged_occupancy(e->kernel[variant], threads, e->warp_bytes[variant]);
     const int per_sm = g.bps > 0 && g.bps < occ ? g.bps : occ;
     const int64_t wpb = threads / 32;
