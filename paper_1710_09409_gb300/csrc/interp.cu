@@ -38,23 +38,44 @@ struct IProg {
   IIns ins[kIMax];
 };
 
-// The register file: real r of register g of this thread.
-template <class M>
+// The register file: real r of register g of this thread, in a slot of SLOT
+// bytes.  The native FP64 path of the range guard runs on the register file of
+// another arithmetic: a double in the thread's own slots, moved as two words
+// where the slot is not aligned to it.
+template <class M, int SLOT = (int)sizeof(typename M::R)>
 struct IRegs {
-  typename M::R* base;
+  using R = typename M::R;
+  unsigned char* base;
   int nt, tid;
-  __device__ __forceinline__ typename M::R& at(int g, int r) const {
-    return base[(g * 18 + r) * nt + tid];
+  __device__ __forceinline__ unsigned char* slot(int g, int r) const {
+    return base + (size_t)((g * 18 + r) * nt + tid) * SLOT;
+  }
+  __device__ __forceinline__ R ld(int g, int r) const {
+    if constexpr (SLOT % alignof(R) == 0) {
+      return *reinterpret_cast<const R*>(slot(g, r));
+    } else {
+      const uint32_t* w = reinterpret_cast<const uint32_t*>(slot(g, r));
+      return u2d(w[0], w[1]);
+    }
+  }
+  __device__ __forceinline__ void st(int g, int r, const R& v) const {
+    if constexpr (SLOT % alignof(R) == 0) {
+      *reinterpret_cast<R*>(slot(g, r)) = v;
+    } else {
+      uint32_t* w = reinterpret_cast<uint32_t*>(slot(g, r));
+      w[0] = (uint32_t)__double2loint(v);
+      w[1] = (uint32_t)__double2hiint(v);
+    }
   }
   template <int W>
-  __device__ __forceinline__ void get(int g, typename M::R* v) const {
+  __device__ __forceinline__ void get(int g, R* v) const {
 #pragma unroll
-    for (int r = 0; r < W; ++r) v[r] = at(g, r);
+    for (int r = 0; r < W; ++r) v[r] = ld(g, r);
   }
   template <int W>
-  __device__ __forceinline__ void put(int g, const typename M::R* v) const {
+  __device__ __forceinline__ void put(int g, const R* v) const {
 #pragma unroll
-    for (int r = 0; r < W; ++r) at(g, r) = v[r];
+    for (int r = 0; r < W; ++r) st(g, r, v[r]);
   }
 };
 
@@ -79,8 +100,8 @@ __device__ __forceinline__ void i_load(const FieldDesc& f, int64_t s, int mu, ty
   M::template normalize_obj<W>(r);
 }
 
-template <class M, int W>
-__device__ __forceinline__ void i_add(const IRegs<M>& R, const IIns& in, int sg) {
+template <class M, int W, class Regs>
+__device__ __forceinline__ void i_add(const Regs& R, const IIns& in, int sg) {
   typename M::R x[W], y[W], d[W];
   typename M::A acc[W];
   R.template get<W>(in.a, x);
@@ -95,8 +116,8 @@ __device__ __forceinline__ void i_add(const IRegs<M>& R, const IIns& in, int sg)
   R.template put<W>(in.dst, d);
 }
 
-template <class M, int W>
-__device__ __forceinline__ void i_scale(const IRegs<M>& R, const IIns& in, const KParams& p) {
+template <class M, int W, class Regs>
+__device__ __forceinline__ void i_scale(const Regs& R, const IIns& in, const KParams& p) {
   typename M::R x[W], d[W];
   typename M::A acc[W];
   R.template get<W>(in.a, x);
@@ -107,8 +128,8 @@ __device__ __forceinline__ void i_scale(const IRegs<M>& R, const IIns& in, const
   R.template put<W>(in.dst, d);
 }
 
-template <class M, int W>
-__device__ __forceinline__ void i_store(const FieldDesc& dst, int64_t s, int mu, const IRegs<M>& R,
+template <class M, int W, class Regs>
+__device__ __forceinline__ void i_store(const FieldDesc& dst, int64_t s, int mu, const Regs& R,
                                         int g) {
   typename M::R z[W];
   R.template get<W>(g, z);
@@ -125,8 +146,8 @@ __device__ __forceinline__ void i_store(const FieldDesc& dst, int64_t s, int mu,
 }
 
 // Run the program on site s into the register file R (g: range guard).
-template <class M>
-__device__ __forceinline__ void i_run(const KParams& p, const IProg& prog, const IRegs<M>& R,
+template <class M, class Regs>
+__device__ __forceinline__ void i_run(const KParams& p, const IProg& prog, const Regs& R,
                                       int64_t s, int mu, uint32_t& g) {
   using Rv = typename M::R;
   using Av = typename M::A;
@@ -202,8 +223,8 @@ __device__ __forceinline__ void i_run(const KParams& p, const IProg& prog, const
   }
 }
 
-template <class M>
-__device__ __forceinline__ void i_store_root(const KParams& p, const IProg& prog, const IRegs<M>& R,
+template <class M, class Regs>
+__device__ __forceinline__ void i_store_root(const KParams& p, const IProg& prog, const Regs& R,
                                              int64_t s, int mu) {
   if (prog.root_kind == KR) i_store<M, 1>(p.dst, s, mu, R, prog.root);
   else if (prog.root_kind == KV) i_store<M, 6>(p.dst, s, mu, R, prog.root);
@@ -211,11 +232,12 @@ __device__ __forceinline__ void i_store_root(const KParams& p, const IProg& prog
 }
 
 // The range guard's path: the program again in native FP64 on this thread's
-// slice of the register file (a double is no wider than any arithmetic's
-// real, so it fits), then the store.  Out of line, off the hot loop.
-__device__ __noinline__ void i_site_f64(const KParams& p, const IProg& prog, void* base, int nt,
+// slots of the register file (a double is no wider than any arithmetic's
+// real, so it fits its slot), then the store.  Out of line, off the hot loop.
+template <int SLOT>
+__device__ __noinline__ void i_site_f64(const KParams& p, const IProg& prog, unsigned char* base, int nt,
                                         int tid, int64_t s, int mu) {
-  const IRegs<MathF64> R{reinterpret_cast<double*>(base), nt, tid};
+  const IRegs<MathF64, SLOT> R{base, nt, tid};
   uint32_t g = 0;
   i_run<MathF64>(p, prog, R, s, mu, g);
   i_store_root<MathF64>(p, prog, R, s, mu);
@@ -226,13 +248,14 @@ __global__ void __launch_bounds__(128) k_interp(const __grid_constant__ KParams 
                                                 const __grid_constant__ IProg prog) {
   using Rv = typename M::R;
   extern __shared__ __align__(16) unsigned char i_smem[];
-  const IRegs<M> R{reinterpret_cast<Rv*>(i_smem), (int)blockDim.x, (int)threadIdx.x};
+  const IRegs<M> R{i_smem, (int)blockDim.x, (int)threadIdx.x};
   const int mu = blockIdx.y;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < p.nvec; s += stride) {
     uint32_t g = p.gscal;
     i_run<M>(p, prog, R, s, mu, g);
-    if (M::kGuard && g >= p.ghi) i_site_f64(p, prog, i_smem, (int)blockDim.x, (int)threadIdx.x, s, mu);
+    if (M::kGuard && g >= p.ghi)
+      i_site_f64<(int)sizeof(Rv)>(p, prog, i_smem, (int)blockDim.x, (int)threadIdx.x, s, mu);
     else i_store_root<M>(p, prog, R, s, mu);
   }
 }
