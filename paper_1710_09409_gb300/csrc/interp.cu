@@ -11,6 +11,7 @@
 // loaded at their first use and every register is freed after its last.
 #include <string.h>
 
+#include <mutex>
 #include <vector>
 
 #include "dev_kernels.cuh"
@@ -27,7 +28,8 @@ struct IIns {
   int8_t op, dst, a, b;
   int8_t w;    // width in reals of the result (18, 6, 1)
   int8_t arg;  // leaf slot (LOAD, with kind in b) / factor index (SCALE)
-  int8_t pad[2];
+  int8_t adj;  // products: 1 the left operand's adjoint, 2 the right one's
+  int8_t pad;
 };
 
 struct IProg {
@@ -35,6 +37,8 @@ struct IProg {
   int32_t root;
   int32_t root_kind;
   int32_t nregs;   // registers the program uses (shared memory is sized to them)
+  int32_t nloads;  // its loads in order: leaf slot and width in reals
+  int8_t load_leaf[kMaxLeaves], load_w[kMaxLeaves];
   IIns ins[kIMax];
 };
 
@@ -100,6 +104,18 @@ __device__ __forceinline__ void i_load(const FieldDesc& f, int64_t s, int mu, ty
   M::template normalize_obj<W>(r);
 }
 
+// A matrix register, or (FOLD and dag) its adjoint.
+template <class M, bool FOLD, class Regs>
+__device__ __forceinline__ void i_get_mat(const Regs& R, int g, bool dag, typename M::R* v) {
+  R.template get<18>(g, v);
+  if (FOLD && dag) {
+    typename M::R t[18];
+    adjoint<M>(t, v);
+#pragma unroll
+    for (int r = 0; r < 18; ++r) v[r] = t[r];
+  }
+}
+
 template <class M, int W, class Regs>
 __device__ __forceinline__ void i_add(const Regs& R, const IIns& in, int sg) {
   typename M::R x[W], y[W], d[W];
@@ -146,7 +162,8 @@ __device__ __forceinline__ void i_store(const FieldDesc& dst, int64_t s, int mu,
 }
 
 // Run the program on site s into the register file R (g: range guard).
-template <class M, class Regs>
+// FOLD: products may read their operands' adjoints (the pair kernel's programs).
+template <class M, bool FOLD, class Regs>
 __device__ __forceinline__ void i_run(const KParams& p, const IProg& prog, const Regs& R,
                                       int64_t s, int mu, uint32_t& g) {
   using Rv = typename M::R;
@@ -171,8 +188,8 @@ __device__ __forceinline__ void i_run(const KParams& p, const IProg& prog, const
       case I_MMUL: {
         Rv x[18], y[18], d[18];
         Av acc[18];
-        R.template get<18>(in.a, x);
-        R.template get<18>(in.b, y);
+        i_get_mat<M, FOLD>(R, in.a, (in.adj & 1) != 0, x);
+        i_get_mat<M, FOLD>(R, in.b, (in.adj & 2) != 0, y);
         mm_acc<M, true, 1, false, false>(acc, x, y);
         finish<M, 18>(d, acc);
         R.template put<18>(in.dst, d);
@@ -181,7 +198,7 @@ __device__ __forceinline__ void i_run(const KParams& p, const IProg& prog, const
       case I_MVMUL: {
         Rv x[18], y[6], d[6];
         Av acc[6];
-        R.template get<18>(in.a, x);
+        i_get_mat<M, FOLD>(R, in.a, (in.adj & 1) != 0, x);
         R.template get<6>(in.b, y);
         mv_acc<M, true, 1, false>(acc, x, y);
         finish<M, 6>(d, acc);
@@ -234,12 +251,12 @@ __device__ __forceinline__ void i_store_root(const KParams& p, const IProg& prog
 // The range guard's path: the program again in native FP64 on this thread's
 // slots of the register file (a double is no wider than any arithmetic's
 // real, so it fits its slot), then the store.  Out of line, off the hot loop.
-template <int SLOT>
+template <int SLOT, bool FOLD>
 __device__ __noinline__ void i_site_f64(const KParams& p, const IProg& prog, unsigned char* base, int nt,
                                         int tid, int64_t s, int mu) {
   const IRegs<MathF64, SLOT> R{base, nt, tid};
   uint32_t g = 0;
-  i_run<MathF64>(p, prog, R, s, mu, g);
+  i_run<MathF64, FOLD>(p, prog, R, s, mu, g);
   i_store_root<MathF64>(p, prog, R, s, mu);
 }
 
@@ -253,10 +270,297 @@ __global__ void __launch_bounds__(128) k_interp(const __grid_constant__ KParams 
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < p.nvec; s += stride) {
     uint32_t g = p.gscal;
-    i_run<M>(p, prog, R, s, mu, g);
+    i_run<M, false>(p, prog, R, s, mu, g);
     if (M::kGuard && g >= p.ghi)
-      i_site_f64<(int)sizeof(Rv)>(p, prog, i_smem, (int)blockDim.x, (int)threadIdx.x, s, mu);
+      i_site_f64<(int)sizeof(Rv), false>(p, prog, i_smem, (int)blockDim.x, (int)threadIdx.x, s, mu);
     else i_store_root<M>(p, prog, R, s, mu);
+  }
+}
+
+// ------------------------------------------- pair arithmetic: two sites per thread
+// The pair arithmetic's interpreter packs every FP32 operation over two sites,
+// s and s + blockDim.x of a run of 2 blockDim.x sites: half the instructions,
+// program steps and operand fetches per site, and no operand is copied,
+// swapped or signed (as in dev_pairs.cuh).  A register's real is 16 bytes per
+// thread ([register][real][thread]: leading parts of both sites, trailing
+// parts), one shared-memory access.  Each lane performs MathDF's operations in
+// MathDF's order: the values are those of the one-site interpreter.
+// The next load's object is fetched while the steps before it run.  Bound by
+// latency at 8 warps per SM (the register file: 864 bytes per thread and three
+// registers): 2,420 instructions per 32 sites (3,490), issue 35%.
+// Measured against one site per thread (both with results in place): a (b + c) -
+// d at 24^4 63.7 / 65.2 us, 28^4 113 / 121, 40^4 440 / 476 (506 before);
+// adj(a) b + c at 40^4 348 / 406.  Programs of four registers run 6 warps and
+// are slower here (a (b c - d) at 40^4 592 / 561), programs of three products
+// and more too (a b c d at 32^4 228 / 223: their rolled rows keep fewer
+// accumulations in flight), and small lattices, a thread's chain being longer.
+constexpr int64_t kPairSites = 300000;
+constexpr int kPairRegs = 3;
+struct PRegs {
+  float4* base;
+  int nt, tid;
+  __device__ __forceinline__ dp get(int g, int r) const {
+    const float4 v = base[(g * 18 + r) * nt + tid];
+    return dp{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+  }
+  __device__ __forceinline__ void put(int g, int r, const dp& v) const {
+    base[(g * 18 + r) * nt + tid] = make_float4(v.h.x, v.h.y, v.l.x, v.l.y);
+  }
+  // element e (of 9) of a matrix register, or of its adjoint
+  __device__ __forceinline__ void get_c(int g, int i, int j, bool dag, dp& re, dp& im) const {
+    const int e = dag ? 3 * j + i : 3 * i + j;
+    re = get(g, 2 * e);
+    im = get(g, 2 * e + 1);
+    const float sg = dag ? -1.0f : 1.0f;   // exact
+    im.h = f2_mul_packed(im.h, make_float2(sg, sg));
+    im.l = f2_mul_packed(im.l, make_float2(sg, sg));
+  }
+};
+
+// accumulator -> operand (MathDF::finish)
+__device__ __forceinline__ dp dp_norm(const dpa& a) {
+  const float2 h = f2_add(a.S, a.lo);
+  return dp{h, f2_sub(a.lo, f2_sub(h, a.S))};
+}
+
+// a + b or a - b of two operands, finished (MathDF::add twice, then finish)
+template <bool NEG>
+__device__ __forceinline__ dp dp_sum(const dp& a, const dp& b) {
+  dpa z{a.h, a.l};
+  df2_combine<NEG ? -1 : 1>(z, dpa{b.h, b.l});
+  return dp_norm(z);
+}
+
+// The raw object of the next load, fetched while the steps before it run: the
+// complex elements of both sites (a real field: its two values in v0[0]).
+struct PNext {
+  uint4 v0[9], v1[9];
+  __device__ __forceinline__ void fetch(const KParams& p, const IProg& prog, int i, int64_t s0, int64_t s1,
+                                        int mu) {
+    const FieldDesc& f = p.leaf[prog.load_leaf[i]];
+    const int w = prog.load_w[i];
+    const int64_t b0 = elem_base(f, s0, mu), b1 = elem_base(f, s1, mu);
+    if (w == 1) {
+      const uint2 a = ld8((const char*)f.ptr + b0 * 8), b = ld8((const char*)f.ptr + b1 * 8);
+      v0[0] = make_uint4(a.x, a.y, b.x, b.y);
+      return;
+    }
+    const char* p0 = (const char*)f.ptr + b0 * 16;
+    const char* p1 = (const char*)f.ptr + b1 * 16;
+#pragma unroll
+    for (int c = 0; c < 9; ++c) {
+      if (c == 3 && w == 6) break;
+      v0[c] = ld16(p0 + c * f.s_c * 16);
+      v1[c] = ld16(p1 + c * f.s_c * 16);
+    }
+  }
+  template <int NC>
+  __device__ __forceinline__ void put(const PRegs& R, int g, uint32_t& gm) const {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      gm = guard_max(guard_max(gm, v0[c].y, v0[c].w), v1[c].y, v1[c].w);
+      R.put(g, 2 * c, dp_split(v0[c].x, v0[c].y, v1[c].x, v1[c].y));
+      R.put(g, 2 * c + 1, dp_split(v0[c].z, v0[c].w, v1[c].z, v1[c].w));
+    }
+  }
+};
+
+// Reals r0 .. r0 + N - 1 of a sum (sg: +-1 of the second operand) and of a scaled
+// operand: all operands first, so that their reads overlap.
+template <int N>
+__device__ __forceinline__ void p_add(const PRegs& R, const IIns& in, int r0, float2 sg) {
+  dp a[N], b[N];
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    a[q] = R.get(in.a, r0 + q);
+    b[q] = R.get(in.b, r0 + q);
+  }
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+    R.put(in.dst, r0 + q, dp_sum<false>(a[q], dp{f2_mul_packed(b[q].h, sg), f2_mul_packed(b[q].l, sg)}));
+}
+template <int N>
+__device__ __forceinline__ void p_scale(const PRegs& R, const IIns& in, int r0, const dp& sc) {
+  dp x[N];
+#pragma unroll
+  for (int q = 0; q < N; ++q) x[q] = R.get(in.a, r0 + q);
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    dpa a;
+    dp_first<false>(a, sc, x[q]);
+    R.put(in.dst, r0 + q, dp_norm(a));
+  }
+}
+
+// The program on sites s0, s1; n0, n1: the sites after them (they are this
+// thread's next ones, or these again), whose first load is fetched ahead.
+__device__ __forceinline__ void p_run(const KParams& p, const IProg& prog, const PRegs& R, PNext& next,
+                                      int64_t s0, int64_t s1, int64_t n0, int64_t n1, int mu, uint32_t& gm) {
+  int loaded = 0;
+  for (int pc = 0; pc < prog.n; ++pc) {
+    const IIns in = prog.ins[pc];
+    switch (in.op) {
+      case I_LOAD: {
+        if (in.w == 18) {
+          next.put<9>(R, in.dst, gm);
+        } else if (in.w == 6) {
+          next.put<3>(R, in.dst, gm);
+        } else {
+          const uint4 v = next.v0[0];
+          gm = guard_max(gm, v.y, v.w);
+          R.put(in.dst, 0, dp_split(v.x, v.y, v.z, v.w));
+        }
+        if (++loaded < prog.nloads) next.fetch(p, prog, loaded, s0, s1, mu);
+        else next.fetch(p, prog, 0, n0, n1, mu);
+        break;
+      }
+      case I_MMUL: {
+        // op(y) held, op(x) and the result one row at a time
+        const bool dx = (in.adj & 1) != 0, dy = (in.adj & 2) != 0;
+        dp y[18];
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+          for (int k = 0; k < 3; ++k) R.get_c(in.b, j, k, dy, y[6 * j + 2 * k], y[6 * j + 2 * k + 1]);
+        dp x[6];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) R.get_c(in.a, 0, j, dx, x[2 * j], x[2 * j + 1]);
+#pragma unroll 1
+        for (int i = 0; i < 3; ++i) {
+          dpa re[3], im[3];
+          dpa* const a[6] = {&re[0], &re[1], &re[2], &im[0], &im[1], &im[2]};
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            const dp xr = x[2 * j], xm = x[2 * j + 1];
+            if (i < 2) R.get_c(in.a, i + 1, j, dx, x[2 * j], x[2 * j + 1]);   // the next row's
+            const dp* const yj = y + 6 * j;
+            const dp* const y0[6] = {yj, yj + 2, yj + 4, yj + 1, yj + 3, yj + 5};
+            const dp* const y1[6] = {yj + 1, yj + 3, yj + 5, yj, yj + 2, yj + 4};
+            if (j == 0) dp_fma_shared<6, true, 0u>(a, xr, y0);
+            else dp_fma_shared<6, false, 0u>(a, xr, y0);
+            dp_fma_shared<6, false, 7u>(a, xm, y1);
+          }
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            R.put(in.dst, 6 * i + 2 * k, dp_norm(re[k]));
+            R.put(in.dst, 6 * i + 2 * k + 1, dp_norm(im[k]));
+          }
+        }
+        break;
+      }
+      case I_MVMUL: {
+        const bool dx = (in.adj & 1) != 0;
+        dp y[6];
+#pragma unroll
+        for (int r = 0; r < 6; ++r) y[r] = R.get(in.b, r);
+#pragma unroll 1
+        for (int i = 0; i < 3; ++i) {
+          dpa re, im;
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            dp xr, xm;
+            R.get_c(in.a, i, j, dx, xr, xm);
+            if (j == 0) dp_cterm<true, 1, false, false>(re, im, xr, xm, y[2 * j], y[2 * j + 1]);
+            else dp_cterm<false, 1, false, false>(re, im, xr, xm, y[2 * j], y[2 * j + 1]);
+          }
+          R.put(in.dst, 2 * i, dp_norm(re));
+          R.put(in.dst, 2 * i + 1, dp_norm(im));
+        }
+        break;
+      }
+      case I_RMUL: {
+        dpa a;
+        dp_first<false>(a, R.get(in.a, 0), R.get(in.b, 0));
+        R.put(in.dst, 0, dp_norm(a));
+        break;
+      }
+      case I_ADD:
+      case I_SUB: {
+        const float sg = in.op == I_ADD ? 1.0f : -1.0f;   // exact
+        const float2 s2 = make_float2(sg, sg);
+        if (in.w == 1) {
+          p_add<1>(R, in, 0, s2);
+        } else {
+#pragma unroll 1
+          for (int r0 = 0; r0 < in.w; r0 += 6) p_add<6>(R, in, r0, s2);
+        }
+        break;
+      }
+      case I_SCALE: {
+        const dp sc{make_float2(p.sch[in.arg], p.sch[in.arg]), make_float2(p.scl[in.arg], p.scl[in.arg])};
+        if (in.w == 1) {
+          p_scale<1>(R, in, 0, sc);
+        } else {
+#pragma unroll 1
+          for (int r0 = 0; r0 < in.w; r0 += 6) p_scale<6>(R, in, r0, sc);
+        }
+        break;
+      }
+      default: {  // I_ADJ
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            dp re, im;
+            R.get_c(in.a, i, j, true, re, im);
+            R.put(in.dst, 2 * (3 * i + j), re);
+            R.put(in.dst, 2 * (3 * i + j) + 1, im);
+          }
+        break;
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ void p_store_root(const KParams& p, const IProg& prog, const PRegs& R,
+                                             int64_t s0, int64_t s1, bool has1, int mu) {
+  char* base = (char*)p.dst.ptr;
+  const int64_t e0 = elem_base(p.dst, s0, mu), e1 = elem_base(p.dst, s1, mu);
+  if (prog.root_kind == KR) {
+    const dp v = R.get(prog.root, 0);
+    double d0, d1;
+    df2_to_double(dpa{v.h, v.l}, d0, d1);
+    st8(base + e0 * 8, make_uint2((uint32_t)__double2loint(d0), (uint32_t)__double2hiint(d0)));
+    if (has1) st8(base + e1 * 8, make_uint2((uint32_t)__double2loint(d1), (uint32_t)__double2hiint(d1)));
+    return;
+  }
+  const int nc = prog.root_kind == KV ? 3 : 9;
+#pragma unroll 1
+  for (int c0 = 0; c0 < nc; c0 += 3) {
+    dp z[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) z[q] = R.get(prog.root, 2 * c0 + q);
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      pair_store_c(base, e0 + (c0 + q) * p.dst.s_c, e1 + (c0 + q) * p.dst.s_c, has1,
+                   dpa{z[2 * q].h, z[2 * q].l}, dpa{z[2 * q + 1].h, z[2 * q + 1].l});
+  }
+}
+
+__global__ void __launch_bounds__(128) k_interp_pair(const __grid_constant__ KParams p,
+                                                     const __grid_constant__ IProg prog) {
+  extern __shared__ __align__(16) unsigned char i_smem[];
+  const int nt = (int)blockDim.x, tid = (int)threadIdx.x;
+  const PRegs R{reinterpret_cast<float4*>(i_smem), nt, tid};
+  const int mu = blockIdx.y;
+  const int64_t step = (int64_t)gridDim.x * 2 * nt;
+  int64_t s0 = (int64_t)blockIdx.x * 2 * nt + tid;
+  if (s0 >= p.nvec) return;
+  PNext next;
+  next.fetch(p, prog, 0, s0, s0 + nt < p.nvec ? s0 + nt : s0, mu);
+  for (; s0 < p.nvec; s0 += step) {
+    const bool has1 = s0 + nt < p.nvec;
+    const int64_t s1 = has1 ? s0 + nt : s0;
+    const int64_t n0 = s0 + step < p.nvec ? s0 + step : s0, n1 = n0 + nt < p.nvec ? n0 + nt : n0;
+    uint32_t gm = p.gscal;
+    p_run(p, prog, R, next, s0, s1, n0, n1, mu, gm);
+    if (gm >= p.ghi) {
+      // native FP64, one site after the other
+      i_site_f64<16, true>(p, prog, i_smem, nt, tid, s0, mu);
+      if (has1) i_site_f64<16, true>(p, prog, i_smem, nt, tid, s1, mu);
+    } else {
+      p_store_root(p, prog, R, s0, s1, has1, mu);
+    }
   }
 }
 
@@ -268,6 +572,8 @@ struct Builder {
   int leaf_reg[kMaxLeaves];
   int uses_left[kMaxLeaves] = {};  // leaf nodes of each slot not generated yet
   const Canon* c;
+  bool reuse = true;  // element-by-element results in place
+  bool fold = true;   // adjoints of a product's operands folded into it
   int nscal = 0;
   int err = 0;
 
@@ -281,11 +587,24 @@ struct Builder {
     err = 1;
     return 0;
   }
+  // whether register r holds a leaf that is still to be used
+  bool kept(int r) const {
+    for (int l = 0; l < kMaxLeaves; ++l)
+      if (leaf_reg[l] == r && uses_left[l] > 0) return true;
+    return false;
+  }
   // free register r unless it holds a leaf that is still to be used
   void release(int r) {
+    if (!kept(r)) busy[r] = false;
+  }
+  // register of an element-by-element result: an operand's own if it is not
+  // needed any more (a leaf's register then holds the leaf no longer)
+  int in_place(int a, int b) {
+    const int d = !reuse ? -1 : !kept(a) ? a : !kept(b) ? b : -1;
+    if (d < 0) return alloc();
     for (int l = 0; l < kMaxLeaves; ++l)
-      if (leaf_reg[l] == r && uses_left[l] > 0) return;
-    busy[r] = false;
+      if (leaf_reg[l] == d) leaf_reg[l] = -1;
+    return d;
   }
   void emit(IIns in) {
     if (prog.n >= kIMax) {
@@ -321,7 +640,11 @@ struct Builder {
           const int r = alloc();
           leaf_reg[l] = r;
           const int kind = e->f->kind;
-          emit(IIns{I_LOAD, (int8_t)r, 0, (int8_t)kind, width(kind), (int8_t)l, {0, 0}});
+          emit(IIns{I_LOAD, (int8_t)r, 0, (int8_t)kind, width(kind), (int8_t)l, 0, 0});
+          if (!err) {
+            prog.load_leaf[prog.nloads] = (int8_t)l;
+            prog.load_w[prog.nloads++] = width(kind);
+          }
         }
         --uses_left[l];
         return leaf_reg[l];
@@ -329,28 +652,35 @@ struct Builder {
       case 4: {
         int k = nscal++;  // factors numbered in the canonical (pre-order) order
         int a = gen(e->a);
-        int d = alloc();
-        emit(IIns{I_SCALE, (int8_t)d, (int8_t)a, 0, width(e->kind), (int8_t)k, {0, 0}});
-        release(a);
+        int d = in_place(a, a);
+        emit(IIns{I_SCALE, (int8_t)d, (int8_t)a, 0, width(e->kind), (int8_t)k, 0, 0});
+        if (a != d) release(a);
         return d;
       }
       case 5: {
         int a = gen(e->a);
         int d = alloc();
-        emit(IIns{I_ADJ, (int8_t)d, (int8_t)a, 0, 18, 0, {0, 0}});
+        emit(IIns{I_ADJ, (int8_t)d, (int8_t)a, 0, 18, 0, 0, 0});
         release(a);
         return d;
       }
       default: {
-        int a = gen(e->a);
-        int b = gen(e->b);
-        int d = alloc();
-        int8_t op;
-        if (e->op == 1) op = e->kind == SU3S_MATRIX ? I_MMUL : e->kind == SU3S_VECTOR ? I_MVMUL : I_RMUL;
-        else op = e->op == 2 ? I_ADD : I_SUB;
-        emit(IIns{op, (int8_t)d, (int8_t)a, (int8_t)b, width(e->kind), 0, {0, 0}});
-        release(a);
-        release(b);
+        const su3s_expr *ea = e->a, *eb = e->b;
+        int8_t adj = 0, op;
+        if (e->op == 1) {
+          op = e->kind == SU3S_MATRIX ? I_MMUL : e->kind == SU3S_VECTOR ? I_MVMUL : I_RMUL;
+          // a product reads the adjoint of an operand from the operand itself
+          for (; fold && ea->op == 5; ea = ea->a) adj ^= 1;
+          for (; fold && eb->op == 5; eb = eb->a) adj ^= 2;
+        } else {
+          op = e->op == 2 ? I_ADD : I_SUB;
+        }
+        int a = gen(ea);
+        int b = gen(eb);
+        int d = e->op == 1 ? alloc() : in_place(a, b);
+        emit(IIns{op, (int8_t)d, (int8_t)a, (int8_t)b, width(e->kind), 0, adj, 0});
+        if (a != d) release(a);
+        if (b != d) release(b);
         return d;
       }
     }
@@ -380,6 +710,45 @@ cudaError_t launch_interp(const KParams& p, const IProg& prog, cudaStream_t st) 
   k_interp<M><<<dim3((unsigned)blocks, (unsigned)p.nmu), threads, smem, st>>>(p, prog);
   return cudaGetLastError();
 }
+
+// Two sites per thread: 288 bytes per register and thread.  The block size with
+// the most warps per SM (the register file in shared memory sets it), larger
+// blocks first.
+cudaError_t launch_interp_pair(const KParams& p, const IProg& prog, cudaStream_t st) {
+  struct Shape {
+    int threads, per_sm;
+  };
+  static std::mutex mu;
+  static Shape shapes[kPairRegs + 1];   // by registers used, looked up once each
+  const size_t per_thread = (size_t)prog.nregs * 18 * sizeof(float4);
+  Shape sh;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    Shape& c = shapes[prog.nregs];
+    if (c.threads == 0) {
+      cudaError_t e = cudaFuncSetAttribute(k_interp_pair, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           smem_optin());
+      Shape best{0, 0};
+      for (int t = 128; t >= 32 && e == cudaSuccess; t -= 32) {
+        if (per_thread * t > (size_t)smem_optin()) continue;
+        int n = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_interp_pair, t, per_thread * t);
+        if (n * t > best.per_sm * best.threads) best = Shape{t, n};
+      }
+      if (e != cudaSuccess) return e;
+      if (best.threads == 0) return cudaErrorInvalidConfiguration;
+      c = best;
+    }
+    sh = c;
+  }
+  const int threads = sh.threads, per_sm = sh.per_sm;
+  int64_t blocks = (int64_t)per_sm * sm_count();               // one wave, grid-stride
+  const int64_t need = (p.nvec + 2 * threads - 1) / (2 * threads);
+  if (blocks > need) blocks = need;
+  if (blocks < 1) blocks = 1;
+  k_interp_pair<<<dim3((unsigned)blocks, (unsigned)p.nmu), threads, per_thread * threads, st>>>(p, prog);
+  return cudaGetLastError();
+}
 }  // namespace
 
 // Degree of a runtime tree (most factors in one term), as Degree<> of the
@@ -398,15 +767,34 @@ static int degree(const su3s_expr* e) {
 }
 
 int interp_eval(const su3s_expr* e, const Canon& c, su3s_field* dest, int math, cudaStream_t st) {
+  // The limits are those of the plain program (one register per result, adjoints
+  // as steps of their own); what runs is never longer.
+  // Two sites per thread from kPairSites on, for programs of at most two products
+  // whose registers let 8 warps per SM run; else one site per thread.
+  const bool large = math == MATH_DF && (int64_t)dest->Vpad * dest->nmu >= kPairSites;
   Builder bld;
-  memset(&bld.prog, 0, sizeof bld.prog);
-  bld.c = &c;
-  for (int l = 0; l < kMaxLeaves; ++l) bld.leaf_reg[l] = -1;
-  bld.count_uses(e);
-  int root = bld.gen(e);
-  if (bld.err)
-    return fail(SU3S_EUNSUPPORTED, "expression too large for the interpreter (%d registers, %d steps)",
-                kIRegs, kIMax);
+  int root = 0;
+  bool pairs = false;
+  for (int pass = 0; pass < 3; ++pass) {
+    // 0: the limits; 1: two sites per thread, adjoints read in place; 2: one site
+    if (pass == 1 && !large) continue;
+    bld = Builder();
+    memset(&bld.prog, 0, sizeof bld.prog);
+    bld.c = &c;
+    bld.reuse = pass > 0;
+    bld.fold = pass == 1;
+    for (int l = 0; l < kMaxLeaves; ++l) bld.leaf_reg[l] = -1;
+    bld.count_uses(e);
+    root = bld.gen(e);
+    if (bld.err)
+      return fail(SU3S_EUNSUPPORTED, "expression too large for the interpreter (%d registers, %d steps)",
+                  kIRegs, kIMax);
+    int products = 0;
+    for (int i = 0; i < bld.prog.n; ++i)
+      products += bld.prog.ins[i].op == I_MMUL || bld.prog.ins[i].op == I_MVMUL;
+    pairs = pass == 1 && bld.prog.nregs <= kPairRegs && products <= 2;
+    if (pairs) break;
+  }
   bld.prog.root = root;
   bld.prog.root_kind = c.kind;
   KParams p;
@@ -414,7 +802,8 @@ int interp_eval(const su3s_expr* e, const Canon& c, su3s_field* dest, int math, 
   p.ghi = guard_hi(degree(e));
   cudaError_t ce = math == MATH_F64  ? launch_interp<MathF64>(p, bld.prog, st)
                    : math == MATH_FX ? launch_interp<MathFX>(p, bld.prog, st)
-                                     : launch_interp<MathDFScalar>(p, bld.prog, st);
+                                     : pairs ? launch_interp_pair(p, bld.prog, st)
+                                               : launch_interp<MathDFScalar>(p, bld.prog, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "interpreter kernel launch");
   return SU3S_OK;
 }
