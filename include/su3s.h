@@ -444,6 +444,35 @@ int su3s_tune_adjoint(const su3s_expr* e, const su3s_field* grad_out, su3s_field
  * EINVAL for other values. */
 int su3s_set_adjoint_split(int mode);
 
+/* A tree over caller-owned FP64 device buffers, in postfix order: one call
+ * builds its fields and nodes, runs and releases them (what su3s_field_wrap,
+ * su3s_expr_* and the calls below do one by one, with the same checks and
+ * results).  prog holds nprog pairs (operation, argument): 0 leaf (argument:
+ * buffer 0..nleaf-1), 1 product, 2 sum, 3 difference of the two values before
+ * it, 4 real factor (argument: 0..nscalar-1) and 5 adjoint of the value before
+ * it; one value remains.  Every buffer has nmu objects per site of its kind in
+ * the layout and block given, and holds at least su3s_field_bytes (leaf_bytes:
+ * its size).  The same buffer listed twice counts as two leaves. */
+typedef struct su3s_tree {
+  const su3s_lattice* lat;
+  const int32_t* prog;
+  const double* scalars;
+  const int* kinds;
+  void* const* leaves;
+  const size_t* leaf_bytes;
+  int nprog, nscalar, nleaf;
+  int nmu, layout, block;
+} su3s_tree;
+
+/* dest = the tree's value at every site (su3s_eval_math). */
+int su3s_tree_eval(const su3s_tree* t, void* dest, size_t dest_bytes, int math, void* stream);
+
+/* Reverse mode (su3s_eval_adjoint): grads[i] receives dL/d(buffer i), NULL
+ * entries and buffers the tree does not read are skipped; each holds
+ * su3s_field_bytes of its buffer's field. */
+int su3s_tree_adjoint(const su3s_tree* t, void* grad_out, size_t grad_out_bytes, void* const* grads,
+                      int math, void* stream);
+
 /* Number of unique leaves of `e` in *n. */
 int su3s_expr_num_leaves(const su3s_expr* e, int* n);
 

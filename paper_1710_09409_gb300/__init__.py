@@ -16,8 +16,10 @@ dest[x] = expr[x] for every site x in one pass (Sec. 4, Listing 3: z = x*y).
 import ctypes
 import numbers
 import os
+import threading
 
 import numpy as np
+import torch
 
 from . import build as _build
 
@@ -30,6 +32,17 @@ PREC_NAMES = {F64: "f64", F32: "f32", BF16: "bf16", F16: "f16", F64_C12: "f64_c1
               F32_C12: "f32_c12"}
 
 _lib = None
+
+
+_leaf_lock = threading.Lock()
+
+
+class _Tree(ctypes.Structure):
+    """su3s_tree: a postfix tree over device buffers (built and released within one call)."""
+    _fields_ = [("lat", ctypes.c_void_p), ("prog", ctypes.c_void_p), ("scalars", ctypes.c_void_p),
+                ("kinds", ctypes.c_void_p), ("leaves", ctypes.c_void_p), ("leaf_bytes", ctypes.c_void_p),
+                ("nprog", ctypes.c_int), ("nscalar", ctypes.c_int), ("nleaf", ctypes.c_int),
+                ("nmu", ctypes.c_int), ("layout", ctypes.c_int), ("block", ctypes.c_int)]
 
 
 class Su3sError(RuntimeError):
@@ -110,6 +123,8 @@ def load(build_if_missing=False):
         "su3s_hop": ([P, P, P, I, P], I),
         "su3s_dslash": ([P, P, P, I, P], I),
         "su3s_set_adjoint_split": ([I], I),
+        "su3s_tree_eval": ([ctypes.POINTER(_Tree), P, SZ, I, P], I),
+        "su3s_tree_adjoint": ([ctypes.POINTER(_Tree), P, SZ, PP, I, P], I),
     }
     for name, (args, res) in sigs.items():
         fn = getattr(L, name)
@@ -124,14 +139,17 @@ def _check(rc):
         raise Su3sError(rc, _lib.su3s_last_error().decode())
 
 
+# cudaStream_t of the current stream of a device, without a torch.cuda.Stream object
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
     """cudaStream_t of a torch stream (None = torch's current stream)."""
-    import torch
     if stream is None:
-        stream = torch.cuda.current_stream()
-    if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
+        return torch.cuda.current_stream().cuda_stream
+    return stream if isinstance(stream, int) else stream.cuda_stream
 
 
 def catalogue():
@@ -203,7 +221,6 @@ class Field:
     """
 
     def __init__(self, lattice, kind=MATRIX, nmu=1, prec=F64, layout=SOA, block=64, tensor=None):
-        import torch
         L = load()
         self.lattice, self.kind, self.nmu, self.prec = lattice, kind, nmu, prec
         self.layout, self.block = layout, (block if layout == AOSOA else 0)
@@ -222,12 +239,27 @@ class Field:
         _check(L.su3s_field_wrap(lattice._h, kind, nmu, prec, layout, block,
                                  ctypes.c_void_p(tensor.data_ptr()), tb, ctypes.byref(h)))
         self._h = h
+        self._leaf = None
         self.tensor = tensor
 
     def __del__(self):
         if getattr(self, "_h", None) and _lib is not None:
+            if self._leaf is not None:
+                _lib.su3s_expr_free(self._leaf)
             _lib.su3s_field_destroy(self._h)
-            self._h = None
+            self._h = self._leaf = None
+
+    def _leaf_node(self):
+        """The field's leaf node, made once: every tree over the field shares it."""
+        if self._leaf is None:
+            h = ctypes.c_void_p()
+            _check(_lib.su3s_expr_leaf(self._h, ctypes.byref(h)))
+            with _leaf_lock:
+                if self._leaf is None:
+                    self._leaf = h
+                    return h
+            _lib.su3s_expr_free(h)
+        return self._leaf
 
     @property
     def canonical_shape(self):
@@ -243,7 +275,6 @@ class Field:
     def upload(self, host, stream=None):
         """Copy a canonical float64 host array (numpy or CPU tensor; pinned for
         an asynchronous copy) into the field."""
-        import torch
         if isinstance(host, np.ndarray):
             arr = np.ascontiguousarray(host, dtype=np.float64)
             ptr, n, keep = arr.ctypes.data, arr.size, arr
@@ -258,7 +289,6 @@ class Field:
     def download(self, out=None, stream=None):
         """Canonical float64 copy of the field on the host (synchronous unless
         `out` is a pinned CPU tensor and a stream is given)."""
-        import torch
         shape = self.canonical_shape
         if out is None:
             res = np.empty(shape, dtype=np.float64)
@@ -274,7 +304,6 @@ class Field:
         """Canonical float64 copy on the host through the library's fixed
         staging array: no device memory is allocated (fields up to 2^21
         doubles; synchronous)."""
-        import torch
         res = np.empty(self.canonical_shape, dtype=np.float64)
         _check(_lib.su3s_field_download_static(self._h, ctypes.c_void_p(res.ctypes.data), res.size,
                                                _stream(stream)))
@@ -293,7 +322,6 @@ class Field:
     @property
     def stored_dtype(self):
         """torch dtype of one stored real of the field."""
-        import torch
         if self.kind == REAL:
             return torch.float64
         return {F64: torch.float64, F64_C12: torch.float64, F32: torch.float32,
@@ -310,7 +338,6 @@ class Field:
     def upload_stored(self, host, stream=None):
         """Copy a stored-format CPU tensor (`stored_shape`, `stored_dtype`; pinned
         for an asynchronous copy) into the field, bytes unchanged."""
-        import torch
         self._check_stored(host)
         _check(_lib.su3s_field_upload_stored(self._h, ctypes.c_void_p(host.data_ptr()),
                                              host.numel() * host.element_size(), _stream(stream)))
@@ -320,7 +347,6 @@ class Field:
     def download_stored(self, out=None, stream=None):
         """The field's stored bytes as a CPU tensor (`stored_shape`, `stored_dtype`);
         synchronous unless `out` is a pinned CPU tensor and a stream is given."""
-        import torch
         sync = out is None
         if out is None:
             out = torch.empty(self.stored_shape, dtype=self.stored_dtype)
@@ -340,7 +366,6 @@ class Field:
 
     def unpack(self, stream=None):
         """Canonical float64 CUDA tensor of the field."""
-        import torch
         out = torch.empty(self.canonical_shape, dtype=torch.float64, device="cuda")
         _check(_lib.su3s_field_unpack(self._h, ctypes.c_void_p(out.data_ptr()), _stream(stream)))
         return out
@@ -350,16 +375,18 @@ class Field:
         return Expr._leaf(self)
 
     def __mul__(self, o):
+        if isinstance(o, (Field, Expr)):
+            return _binary(_lib.su3s_expr_mul, self, o)
         return self.expr() * o
 
     def __rmul__(self, o):
         return o * self.expr()
 
     def __add__(self, o):
-        return self.expr() + o
+        return _binary(_lib.su3s_expr_add, self, o)
 
     def __sub__(self, o):
-        return self.expr() - o
+        return _binary(_lib.su3s_expr_sub, self, o)
 
     def __neg__(self):
         return -self.expr()
@@ -376,6 +403,23 @@ def _as_expr(x):
     raise TypeError("expected a Field or an Expr, got %r" % (type(x),))
 
 
+def _operand(x):
+    """(node, leaf fields) of a Field or an Expr."""
+    if isinstance(x, Expr):
+        return x._h, x.fields
+    if isinstance(x, Field):
+        return x._leaf_node(), [x]
+    raise TypeError("expected a Field or an Expr, got %r" % (type(x),))
+
+
+def _binary(fn, x, y):
+    hx, fx = _operand(x)
+    hy, fy = _operand(y)
+    h = ctypes.c_void_p()
+    _check(fn(hx, hy, ctypes.byref(h)))
+    return Expr(h, fx + fy)
+
+
 class Expr:
     """Immutable expression tree node (owns one reference to its C handle)."""
 
@@ -389,27 +433,23 @@ class Expr:
         _check(_lib.su3s_expr_leaf(f._h, ctypes.byref(h)))
         return cls(h, [f])
 
-    def _bin(self, fn, other):
-        other = _as_expr(other)
-        h = ctypes.c_void_p()
-        _check(fn(self._h, other._h, ctypes.byref(h)))
-        return Expr(h, self.fields + other.fields)
-
     def __mul__(self, o):
+        if isinstance(o, (Field, Expr)):
+            return _binary(_lib.su3s_expr_mul, self, o)
         if isinstance(o, numbers.Real):
             return self._scale(float(o))
-        return self._bin(_lib.su3s_expr_mul, o)
+        return _binary(_lib.su3s_expr_mul, self, o)
 
     def __rmul__(self, o):
         if isinstance(o, numbers.Real):
             return self._scale(float(o))
-        return _as_expr(o)._bin(_lib.su3s_expr_mul, self)
+        return _binary(_lib.su3s_expr_mul, o, self)
 
     def __add__(self, o):
-        return self._bin(_lib.su3s_expr_add, o)
+        return _binary(_lib.su3s_expr_add, self, o)
 
     def __sub__(self, o):
-        return self._bin(_lib.su3s_expr_sub, o)
+        return _binary(_lib.su3s_expr_sub, self, o)
 
     def __neg__(self):
         return self._scale(-1.0)
@@ -450,8 +490,8 @@ class Expr:
 # -------------------------------------------------------------- evaluation
 def evaluate(dest, expr, math=MATH_DEFAULT, stream=None):
     """dest = expr at every site, one pass, asynchronous on `stream`."""
-    expr = _as_expr(expr)
-    _check(_lib.su3s_eval_math(dest._h, expr._h, math, _stream(stream)))
+    node = _operand(expr)[0]
+    _check(_lib.su3s_eval_math(dest._h, node, math, _stream(stream)))
     return dest
 
 
@@ -498,7 +538,6 @@ def tune_adjoint(expr, grad_out, grads, math=MATH_DEFAULT, stream=None):
 def redot(x, y, out=None, stream=None):
     """sum over all reals of x*y (= sum_x Re tr(X^dagger Y)) as a 1-element
     float64 CUDA tensor."""
-    import torch
     if out is None:
         out = torch.empty(1, dtype=torch.float64, device="cuda")
     _check(_lib.su3s_field_redot(x._h, y._h, ctypes.c_void_p(out.data_ptr()), _stream(stream)))

@@ -432,6 +432,13 @@ static void encode_tmap(su3s_field* f) {
   if (f->layout == SU3S_AOSOA && f->block < 32) return;
   EncodeTiledFn enc = encode_tiled();
   if (!enc) return;
+  // The encoder needs a current context.  A thread that has made no runtime call
+  // yet has none (fields made there had no map and ran the plain-load kernels).
+  static thread_local bool have_context = false;
+  if (!have_context) {
+    int dev = 0;
+    have_context = cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess;
+  }
   const uint64_t w = (uint64_t)f->desc.s_c;
   const uint64_t rows = (uint64_t)f->Vpad * f->nmu * f->ncomp / w;
   // tensor-copy coordinates are signed 32-bit: column 2*site (box end 2*w-1)
@@ -648,20 +655,22 @@ SU3S_EXPORT int su3s_field_bytes(const su3s_lattice* lat, int kind, int nmu, int
   return ok();
 }
 
-SU3S_EXPORT int su3s_field_wrap(const su3s_lattice* lat, int kind, int nmu, int prec, int layout,
-                                int block, void* dev_ptr, size_t bytes, su3s_field** out) {
-  if (!out) return fail(SU3S_EINVAL, "null output handle");
-  *out = nullptr;
-  size_t need = 0;
-  int rc = su3s_field_bytes(lat, kind, nmu, prec, layout, block, &need);
+// The checks of a field over device memory (need: the bytes it takes), and its
+// description.
+static int check_field(const su3s_lattice* lat, int kind, int nmu, int prec, int layout, int block,
+                       const void* dev_ptr, size_t bytes, size_t* need) {
+  const int rc = su3s_field_bytes(lat, kind, nmu, prec, layout, block, need);
   if (rc) return rc;
   if (!dev_ptr) return fail(SU3S_EINVAL, "null device pointer");
   if (((uintptr_t)dev_ptr) & 15) return fail(SU3S_EINVAL, "device pointer is not 16-byte aligned");
-  if (bytes < need)
+  if (bytes < *need)
     return fail(SU3S_ESHAPE, "buffer of %zu bytes is smaller than the %zu the field needs", bytes,
-                need);
-  su3s_field* f = new (std::nothrow) su3s_field;
-  if (!f) return fail(SU3S_ENOMEM, "out of host memory");
+                *need);
+  return SU3S_OK;
+}
+
+static void fill_field(su3s_field* f, const su3s_lattice* lat, int kind, int nmu, int prec, int layout,
+                       int block, void* dev_ptr, size_t bytes) {
   memcpy(f->L, lat->L, sizeof f->L);
   f->V = lat->V;
   f->Vpad = vpad_of(lat->V, layout, block);
@@ -676,6 +685,18 @@ SU3S_EXPORT int su3s_field_wrap(const su3s_lattice* lat, int kind, int nmu, int 
   f->bytes = bytes;
   fill_desc(f);
   encode_tmap(f);
+}
+
+SU3S_EXPORT int su3s_field_wrap(const su3s_lattice* lat, int kind, int nmu, int prec, int layout,
+                                int block, void* dev_ptr, size_t bytes, su3s_field** out) {
+  if (!out) return fail(SU3S_EINVAL, "null output handle");
+  *out = nullptr;
+  size_t need = 0;
+  int rc = check_field(lat, kind, nmu, prec, layout, block, dev_ptr, bytes, &need);
+  if (rc) return rc;
+  su3s_field* f = new (std::nothrow) su3s_field;
+  if (!f) return fail(SU3S_ENOMEM, "out of host memory");
+  fill_field(f, lat, kind, nmu, prec, layout, block, dev_ptr, bytes);
   // Field creation may allocate: resolve here, on the current device, the
   // static staging array of su3s_field_download_static (which loads the
   // module holding it), so that the download itself never has to.  A failure
@@ -847,8 +868,9 @@ SU3S_EXPORT int su3s_expr_adj(const su3s_expr* x, su3s_expr** out) {
   return new_node(5, SU3S_MATRIX, x, nullptr, nullptr, 0.0, out);
 }
 
-SU3S_EXPORT int su3s_expr_free(su3s_expr* e) {
-  // iterative release of a reference-counted DAG
+// Iterative release of a reference-counted DAG (the thread's error message
+// stays).
+static void release_nodes(const su3s_expr* e) {
   std::vector<const su3s_expr*> todo;
   if (e) todo.push_back(e);
   while (!todo.empty()) {
@@ -860,6 +882,10 @@ SU3S_EXPORT int su3s_expr_free(su3s_expr* e) {
       delete n;
     }
   }
+}
+
+SU3S_EXPORT int su3s_expr_free(su3s_expr* e) {
+  release_nodes(e);
   return ok();
 }
 
@@ -1304,4 +1330,104 @@ SU3S_EXPORT int su3s_tune_adjoint(const su3s_expr* e, const su3s_field* gout,
   if (variant_out) *variant_out = var;
   if (best_ms) *best_ms = ms;
   return ok();
+}
+
+// ------------------------------------------------- trees over device memory
+namespace su3s {
+
+// A tree in postfix order over FP64 buffers: fields and nodes live for one call.
+struct TreeCall {
+  std::vector<su3s_field> fields;     // one per buffer
+  std::vector<su3s_expr*> stack;      // nodes not yet taken by a parent
+  ~TreeCall() {
+    for (const su3s_expr* e : stack) release_nodes(e);
+  }
+  int field(const su3s_lattice* lat, int kind, int nmu, int layout, int block, void* p, size_t bytes,
+            su3s_field* f) const {
+    size_t need = 0;
+    const int rc = check_field(lat, kind, nmu, SU3S_F64, layout, block, p, bytes, &need);
+    if (!rc) fill_field(f, lat, kind, nmu, SU3S_F64, layout, block, p, bytes);
+    return rc;
+  }
+  int build(const su3s_tree* t) {
+    if (!t || !t->lat || !t->prog || t->nprog < 1 || t->nleaf < 1 || !t->kinds || !t->leaves ||
+        !t->leaf_bytes)
+      return fail(SU3S_EINVAL, "null argument");
+    fields.resize((size_t)t->nleaf);
+    for (int i = 0; i < t->nleaf; ++i) {
+      const int rc = field(t->lat, t->kinds[i], t->nmu, t->layout, t->block, t->leaves[i],
+                           t->leaf_bytes[i], &fields[(size_t)i]);
+      if (rc) return rc;
+    }
+    stack.reserve((size_t)t->nprog);
+    for (int k = 0; k < t->nprog; ++k) {
+      const int op = t->prog[2 * k], arg = t->prog[2 * k + 1];
+      const size_t need = op == 0 ? 0 : op <= 3 ? 2 : 1, n = stack.size();
+      if (op < 0 || op > 5 || n < need) return fail(SU3S_EINVAL, "bad program at step %d", k);
+      if (op == 0 && (arg < 0 || arg >= t->nleaf)) return fail(SU3S_EINVAL, "leaf %d of %d", arg, t->nleaf);
+      if (op == 4 && (arg < 0 || arg >= t->nscalar || !t->scalars))
+        return fail(SU3S_EINVAL, "real factor %d of %d", arg, t->nscalar);
+      su3s_expr *x = need ? stack[n - need] : nullptr, *y = need == 2 ? stack[n - 1] : nullptr, *e = nullptr;
+      const int rc = op == 0   ? su3s_expr_leaf(&fields[(size_t)arg], &e)
+                     : op == 1 ? su3s_expr_mul(x, y, &e)
+                     : op == 2 ? su3s_expr_add(x, y, &e)
+                     : op == 3 ? su3s_expr_sub(x, y, &e)
+                     : op == 4 ? su3s_expr_scale(t->scalars[arg], x, &e)
+                               : su3s_expr_adj(x, &e);
+      if (rc) return rc;
+      stack.resize(n - need);
+      stack.push_back(e);
+      if (x) release_nodes(x);   // the parent holds them
+      if (y) release_nodes(y);
+    }
+    return stack.size() == 1 ? SU3S_OK : fail(SU3S_EINVAL, "program leaves %zu values", stack.size());
+  }
+};
+
+}  // namespace su3s
+
+SU3S_EXPORT int su3s_tree_eval(const su3s_tree* t, void* dest, size_t dest_bytes, int math, void* stream) {
+  try {
+    TreeCall c;
+    int rc = c.build(t);
+    if (rc) return rc;
+    if (!valid_math(math)) return fail(SU3S_EINVAL, "bad arithmetic %d", math);
+    su3s_field d;
+    rc = c.field(t->lat, c.stack[0]->kind, t->nmu, t->layout, t->block, dest, dest_bytes, &d);
+    if (rc) return rc;
+    return do_eval(&d, c.stack[0], math, (cudaStream_t)stream);
+  } catch (const std::bad_alloc&) {
+    return fail(SU3S_ENOMEM, "out of host memory");
+  }
+}
+
+SU3S_EXPORT int su3s_tree_adjoint(const su3s_tree* t, void* grad_out, size_t grad_out_bytes,
+                                  void* const* grads, int math, void* stream) {
+  try {
+    TreeCall c;
+    int rc = c.build(t);
+    if (rc) return rc;
+    if (!grads) return fail(SU3S_EINVAL, "null argument");
+    su3s_field g;
+    rc = c.field(t->lat, c.stack[0]->kind, t->nmu, t->layout, t->block, grad_out, grad_out_bytes, &g);
+    if (rc) return rc;
+    Canon canon;
+    rc = canonicalize(c.stack[0], &canon);
+    if (rc) return rc;
+    // gradients by buffer -> by unique leaf in order of first appearance
+    std::vector<su3s_field> gf(canon.leaves.size());
+    std::vector<su3s_field*> gp(canon.leaves.size());
+    for (size_t k = 0; k < canon.leaves.size(); ++k) {
+      const size_t i = (size_t)(canon.leaves[k] - c.fields.data());
+      if (!grads[i]) continue;
+      size_t bytes = 0;
+      rc = su3s_field_bytes(t->lat, t->kinds[i], t->nmu, SU3S_F64, t->layout, t->block, &bytes);
+      if (!rc) rc = c.field(t->lat, t->kinds[i], t->nmu, t->layout, t->block, grads[i], bytes, &gf[k]);
+      if (rc) return rc;
+      gp[k] = &gf[k];
+    }
+    return su3s_eval_adjoint(c.stack[0], &g, gp.data(), (int)gp.size(), math, stream);
+  } catch (const std::bad_alloc&) {
+    return fail(SU3S_ENOMEM, "out of host memory");
+  }
 }
