@@ -71,8 +71,8 @@ MATH_ERR = {"fx": "7.8e-16 - 1.6e-15",
 # template arguments name it: (tree, arithmetic type, storage, reverse mode).
 # With the data movement the row ran with (the tuner's variant, else the
 # library's default) this gives the kernel ncu names; the reverse mode of
-# a*b+c*d runs split (two launches of the single-product reverse kernel) when
-# the tuner chose that (reported variant 10 + the halves' variant).
+# a*b+c*d runs split (reported variant 10 + the halves' variant): 14 is both
+# products in one launch, others two launches of the single-product kernel.
 T_MM = "Mul<LM<0>, LM<1>>"
 T_E1 = "Add<Mul<LM<0>, LM<1>>, Mul<LM<2>, LM<3>>>"
 ROW_TREE = {
@@ -132,6 +132,8 @@ def row_launches(r, tuned_variant):
         return r.name, 1, r.nbytes
     tree, math, prec, adj = ROW_TREE[r.name]
     v = tuned_variant if tuned_variant is not None else ROW_DEFAULT_VARIANT.get(r.name, 1)
+    if adj and v == 14:   # both products in one launch, dL/dZ read from HBM once
+        return "k_adjoint_pair_sum<%s>" % T_MM, 1, r.nbytes
     if adj and v >= 10:
         return ADJ_KERNEL[v - 10].format(t=T_MM, m="MathDF"), 2, B_ADJ_MM * r.sites
     names = ADJ_KERNEL if adj else FWD_KERNEL

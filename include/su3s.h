@@ -427,10 +427,11 @@ int su3s_eval_adjoint(const su3s_expr* e, const su3s_field* grad_out, su3s_field
  * timing), result as for su3s_tune; later su3s_eval_adjoint calls on fields
  * of this shape use the fastest geometry.  For a sum or difference of two
  * products of four distinct leaves (a*b + c*d, a*b - c*d, s0 a*b + s1 c*d) it
- * also times the reverse mode split into two single-product launches,
- * (a, b, grad_out -> dA, dB) then (c, d, grad_out -> dC, dD), which read
- * grad_out twice but hold the operands of one product at a time, and keeps
- * the faster form for later calls (a split choice is reported as
+ * also times the reverse mode split into two single-product passes,
+ * (a, b, grad_out -> dA, dB) and (c, d, grad_out -> dC, dD), which read
+ * grad_out twice but hold the operands of one product at a time (two launches,
+ * or one launch of both for a*b + c*d), and keeps the fastest form for later
+ * calls (a split choice is reported as
  * *variant = 10 + the halves' data-movement variant).  Untuned calls of such
  * trees run split. */
 int su3s_tune_adjoint(const su3s_expr* e, const su3s_field* grad_out, su3s_field* const* grad_leaves,

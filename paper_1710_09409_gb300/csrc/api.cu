@@ -78,6 +78,7 @@ static std::map<std::pair<std::string, int>, EvalEntry>& adj_reg() {
 
 static EvalEntry make_entry(const Variants& v, int vps) {
   EvalEntry e{};
+  e.sum_fn = v.sum_fn;
   for (int i = 0; i < kNumVariants; ++i) {
     e.fn[i] = v.fn[i];
     e.kernel[i] = v.kernel[i];
@@ -1147,10 +1148,13 @@ static int prepare_adjoint(const su3s_expr* e, const su3s_field* gout, su3s_fiel
 
 // Reverse mode of a sum or difference of two products of distinct leaves
 // (a*b + c*d, a*b - c*d, s0 a*b + s1 c*d) as two single-product reverse-mode
-// launches, (a, b, dL/dZ -> dA, dB) and (c, d, dL/dZ -> dC, dD).  Each launch
-// reads dL/dZ, so the split moves one object more per site (1,440 instead of
-// 1,296 B per site in FP64), but each kernel holds the operands of one
-// product only.  su3s_tune_adjoint times both forms and keeps the faster.
+// passes, (a, b, dL/dZ -> dA, dB) and (c, d, dL/dZ -> dC, dD).  Each pass
+// reads dL/dZ, one object more per site than the fused kernel, but holds the
+// operands of one product only.  a*b + c*d runs both passes side by side in one
+// launch (k_adjoint_pair_sum), where the second read comes from L2; the others
+// are two launches.  su3s_tune_adjoint times the forms and keeps the fastest.
+constexpr int kSumThreads = 256;   // block of the one-launch form
+
 struct SplitAdjoint {
   GParams p[2];
   const EvalEntry* ent[2];
@@ -1199,30 +1203,58 @@ static bool plan_split_adjoint(const su3s_expr* e, const su3s_field* gout,
   return true;
 }
 
-// Whether the reverse mode of a tree, arithmetic and shape runs split (set by
-// su3s_tune_adjoint; absent: kSplitDefault).
+// How the reverse mode of such a tree, arithmetic and shape runs (set by
+// su3s_tune_adjoint; absent: kSplitSum): one fused pass, one launch per
+// product, or both products in one launch where there is such a kernel
+// (launch_split).
+enum { kFused = 0, kSplit = 1, kSplitSum = 2 };
 static std::mutex g_adj_mode_mu;
-static std::map<std::tuple<std::string, int, int64_t, int>, bool>& adj_mode() {
-  static std::map<std::tuple<std::string, int, int64_t, int>, bool> m;
+static std::map<std::tuple<std::string, int, int64_t, int>, int>& adj_mode() {
+  static std::map<std::tuple<std::string, int, int64_t, int>, int> m;
   return m;
 }
-static constexpr bool kSplitDefault = true;
 
-// -1: tuned choice (or kSplitDefault); 0: always fused; 1: always split
+// -1: tuned choice (or kSplitSum); 0: always fused; 1: always split
 static std::atomic<int> g_split_pref{-1};
 
-static bool use_split(const std::string& sig, int m, int64_t nvec, int nmu) {
+static int split_mode(const std::string& sig, int m, int64_t nvec, int nmu) {
   const int pref = g_split_pref.load(std::memory_order_relaxed);
-  if (pref >= 0) return pref == 1;
+  if (pref >= 0) return pref == 1 ? kSplitSum : kFused;
   std::lock_guard<std::mutex> lk(g_adj_mode_mu);
   auto it = adj_mode().find(std::make_tuple(sig, m, nvec, nmu));
-  return it == adj_mode().end() ? kSplitDefault : it->second;
+  return it == adj_mode().end() ? kSplitSum : it->second;
 }
 
 static cudaError_t launch_planned(const EvalEntry* ent, const GParams& p, bool tma, cudaStream_t st) {
   Launch L;
   plan_launch(ent, p.k.nvec, p.k.nmu, tma, &L);
   return L.fn(&p, L.grid, L.block, st);
+}
+
+// The two products of a split reverse mode.  Both in one launch (kSplitSum)
+// needs the same kernel for both, staged fields, no other pipeline preferred
+// and two units for every warp that a product gets (one block of 8 warps on half
+// the SMs).  18^4 (1.35 units per warp of the chip): 43.8 us in two launches,
+// 30.9 in one.  16^4 (0.84) stays below the line: the two launches' smaller
+// blocks spread its tiles over more SMs (24.7 us).
+static cudaError_t launch_split(const SplitAdjoint& sp, int mode, cudaStream_t st) {
+  const EvalEntry* e = sp.ent[0];
+  const int pref = g_pipeline_pref.load(std::memory_order_relaxed);
+  const int64_t nvec = sp.p[0].k.nvec, units = (nvec / 32 + 1) / 2;
+  const int wpb = kSumThreads / 32, nmu = sp.p[0].k.nmu;
+  if (mode == kSplitSum && e->sum_fn && sp.ent[1] == e && sp.tma[0] && sp.tma[1] && nvec % 32 == 0 &&
+      (pref < 0 || pref == 4) && units * nmu >= (int64_t)wpb * sm_count()) {
+    GParamsSum both;
+    both.half[0] = sp.p[0];
+    both.half[1] = sp.p[1];
+    // one block per SM in all, an even number for every link
+    int nb = (sm_count() + nmu - 1) / nmu;
+    nb += nb & 1;
+    return e->sum_fn(&both, dim3((unsigned)nb, (unsigned)nmu, 1), dim3(kSumThreads, 1, 1), st);
+  }
+  cudaError_t ce = launch_planned(sp.ent[0], sp.p[0], sp.tma[0], st);
+  if (ce == cudaSuccess) ce = launch_planned(sp.ent[1], sp.p[1], sp.tma[1], st);
+  return ce;
 }
 
 SU3S_EXPORT int su3s_set_adjoint_split(int mode) {
@@ -1243,10 +1275,9 @@ SU3S_EXPORT int su3s_eval_adjoint(const su3s_expr* e, const su3s_field* gout,
   canonicalize(e, &c);
   SplitAdjoint sp;
   cudaError_t ce;
-  if (use_split(c.sig, math_for(SU3S_F64, math), p.k.nvec, p.k.nmu) &&
-      plan_split_adjoint(e, gout, gleaves, math, &sp)) {
-    ce = launch_planned(sp.ent[0], sp.p[0], sp.tma[0], st);
-    if (ce == cudaSuccess) ce = launch_planned(sp.ent[1], sp.p[1], sp.tma[1], st);
+  const int mode = split_mode(c.sig, math_for(SU3S_F64, math), p.k.nvec, p.k.nmu);
+  if (mode != kFused && plan_split_adjoint(e, gout, gleaves, math, &sp)) {
+    ce = launch_split(sp, mode, st);
   } else {
     ce = launch_planned(ent, p, tma, st);
   }
@@ -1255,7 +1286,7 @@ SU3S_EXPORT int su3s_eval_adjoint(const su3s_expr* e, const su3s_field* gout,
 }
 
 // Best of two runs of three launches of both halves of a split reverse mode.
-static int time_split(const SplitAdjoint& sp, cudaStream_t st, float* ms_out) {
+static int time_split(const SplitAdjoint& sp, int mode, cudaStream_t st, float* ms_out) {
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess) return fail(SU3S_ECUDA, "event creation failed");
   if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -1266,10 +1297,7 @@ static int time_split(const SplitAdjoint& sp, cudaStream_t st, float* ms_out) {
   cudaError_t ce = cudaSuccess;
   for (int trial = 0; trial < 3 && ce == cudaSuccess; ++trial) {  // trial 0 warms up
     ce = cudaEventRecord(e0, st);
-    for (int r = 0; r < 3 && ce == cudaSuccess; ++r) {
-      ce = launch_planned(sp.ent[0], sp.p[0], sp.tma[0], st);
-      if (ce == cudaSuccess) ce = launch_planned(sp.ent[1], sp.p[1], sp.tma[1], st);
-    }
+    for (int r = 0; r < 3 && ce == cudaSuccess; ++r) ce = launch_split(sp, mode, st);
     if (ce == cudaSuccess) ce = cudaEventRecord(e1, st);
     if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
     float t = 0.f;
@@ -1310,19 +1338,20 @@ SU3S_EXPORT int su3s_tune_adjoint(const su3s_expr* e, const su3s_field* gout,
     if (!rc && sp.ent[1] != sp.ent[0])
       rc = tune_entry(sp.ent[1], &sp.p[1], p.k.nvec, p.k.nmu, sp.tma[1], st, nullptr, nullptr,
                       nullptr, &ms_half);
-    float ms_split = 0.f;
-    if (!rc) rc = time_split(sp, st, &ms_split);
+    float ms_split = 0.f, ms_sum = 0.f;
+    if (!rc) rc = time_split(sp, kSplit, st, &ms_split);
+    if (!rc) rc = time_split(sp, kSplitSum, st, &ms_sum);
     if (rc) return rc;
-    const bool split = ms_split < ms;
+    const bool split = ms_split < ms || ms_sum < ms, sum = ms_sum < ms_split;
     {
       std::lock_guard<std::mutex> lk(g_adj_mode_mu);
-      adj_mode()[std::make_tuple(c.sig, m, p.k.nvec, p.k.nmu)] = split;
+      adj_mode()[std::make_tuple(c.sig, m, p.k.nvec, p.k.nmu)] = !split ? kFused : sum ? kSplitSum : kSplit;
     }
     if (split) {
-      th = th2;
-      bps = bps2;
-      var = 10 + var2;
-      ms = ms_split;
+      th = sum ? kSumThreads : th2;
+      bps = sum ? 1 : bps2;
+      var = 10 + (sum ? 4 : var2);
+      ms = sum ? ms_sum : ms_split;
     }
   }
   if (threads_out) *threads_out = th;

@@ -1716,12 +1716,28 @@ cudaError_t launch_adjoint_pair(const void* params, dim3 grid, dim3 block, cudaS
   return cudaGetLastError();
 }
 
+template <class Tree>
+cudaError_t launch_adjoint_pair_sum(const void* params, dim3 grid, dim3 block, cudaStream_t st) {
+  constexpr int S = PairAdjLayout::STRIDE;
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(k_adjoint_pair_sum<Tree>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         staged_smem_max(S));
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  k_adjoint_pair_sum<Tree><<<grid, block, (block.x / 32) * S, st>>>(*static_cast<const GParamsSum*>(params));
+  return cudaGetLastError();
+}
+
 // Kernel variants of one tree: 0 plain loads, 1 TMA-staged eagerly (whole
 // tile), 2 TMA-staged lazily (per leaf), 3 TMA-staged through a ring of
 // buffers (trees that read each object once), 4 TMA-staged two tiles at a
 // time with two sites per lane (the pair arithmetic on products of matrix
 // leaves).  1-4 exist for FP64 storage.
 struct Variants {
+  LaunchFn sum_fn;      // reverse mode of a sum of two such products in one launch, or null
   LaunchFn fn[5];
   const void* kernel[5];
   int warp_bytes[5];  // shared memory per warp (0 for plain loads)
@@ -1781,6 +1797,7 @@ void reg_adjoint(int math) {
   if constexpr (pair_adjoint_ok<Tree, M>()) {
     v.fn[4] = &launch_adjoint_pair<Tree>;
     v.kernel[4] = (const void*)&k_adjoint_pair<Tree>;
+    if constexpr (std::is_same<Tree, Mul<LM<0>, LM<1>>>::value) v.sum_fn = &launch_adjoint_pair_sum<Tree>;
     v.warp_bytes[4] = PairAdjLayout::STRIDE;
   }
   constexpr DefaultGeo g = default_geometry<Tree, M, P_F64, true>();

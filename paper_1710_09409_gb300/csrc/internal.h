@@ -64,6 +64,7 @@ int sm_count();
 // 3 TMA-staged ring, 4 TMA-staged two tiles with two sites per lane.
 constexpr int kNumVariants = 5;
 struct EvalEntry {
+  cudaError_t (*sum_fn)(const void*, dim3, dim3, cudaStream_t);  // see Variants
   cudaError_t (*fn[kNumVariants])(const void*, dim3, dim3, cudaStream_t);
   const void* kernel[kNumVariants];
   int warp_bytes[kNumVariants];  // shared memory per warp of the staged variants

@@ -60,3 +60,35 @@ def test_commutator_in_place(su3s):
     su3s.evaluate(z, a.adj() * b - b * a.adj())
     su3s.evaluate(a, a.adj() * b - b * a.adj())
     assert torch.equal(a.tensor, z.tensor)
+
+
+@pytest.mark.parametrize("tiles,nmu,layout,block", [(2431, 1, 0, 64), (2432, 1, 0, 64), (2433, 1, 1, 32),
+                                                    (4865, 1, 0, 64), (811, 3, 0, 64)])
+@pytest.mark.parametrize("skip", [None, 0, 3])
+def test_reverse_mode_of_a_sum_in_one_launch(su3s, tiles, nmu, layout, block, skip):
+    """Both products side by side (from 8 units of two tiles per SM on): the
+    gradients of the fused pass, an odd number of tiles and gradients that are not wanted among
+    them."""
+    lat = su3s.Lattice((32, tiles, 1, 1))
+    g = torch.Generator(device="cuda").manual_seed(13)
+    f = [su3s.Field(lat, su3s.MATRIX, nmu, su3s.F64, layout, block) for _ in range(5)]
+    for x in f:
+        x.pack(torch.randn(x.canonical_shape, dtype=torch.float64, device="cuda", generator=g))
+    a, b, c, d, w = f
+    got = {}
+    for mode in (-1, 0):
+        out = [a.like() for _ in range(4)]
+        for x in out:
+            x.tensor.fill_(7.0)
+        su3s.set_adjoint_split(mode)
+        try:
+            su3s.eval_adjoint(a * b + c * d, w, [None if k == skip else x for k, x in enumerate(out)])
+        finally:
+            su3s.set_adjoint_split(-1)
+        got[mode] = out
+    for k in range(4):
+        if k == skip:
+            assert got[-1][k].tensor.eq(7.0).all()
+        else:
+            assert torch.equal(got[-1][k].unpack(), got[0][k].unpack()), k
+    assert su3s.device_error() == 0
