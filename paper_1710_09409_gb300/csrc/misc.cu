@@ -196,47 +196,65 @@ __device__ __forceinline__ void zmul(double& ar, double& ai, double br, double b
   ar = re;
 }
 
-// The same projection with fewer FP64 operations (the FP64 pipe bounds the
-// kernel: 91% busy; 2.59 M FP64 matrices 1,989 -> 1,024 us against the sweeps
-// and FP64 atan2 and sincos of the definition, which stay for the cases below;
-// errors against extended precision, near-unitary input: 4.6e-17 rms, 3.9e-16
-// at most, the definition's 4.3e-17 and 3.2e-16).  Rows 0 and 1 as in the definition.  Of row 2 only a phase is free:
-// orthonormal to rows 0 and 1 it is e^{i alpha} w, w = conj(r0 x r1), so
-// Gram-Schmidt's two sweeps and normalisation come down to the direction of
-// d = <w, row 2>, and e^{i alpha} = d/|d| is also the determinant.  Dividing by
-// its principal cube root leaves rows 0, 1 times q and w times conj(q)^2,
-// q = e^{-i alpha/3}.  q is formed in FP32 (atan2f, sincosf: the branch of
-// the cube root is that of the signs of d) and refined by one step on q^3 d/|d|
-// = 1: with q^3 d/|d| = 1 + z, |z| < 1e-6, q (1 - z/3 + 2/9 z^2) is exact to
-// z^3 < 1e-18.  Returns false where a norm is NaN, zero, or so large or small
-// that it could overflow or underflow here and not in the definition.
+// The part of row b along row a (not normalised; rn = 1/|a|^2) taken out of b:
+// one Gram-Schmidt sweep.  Returns that part's squared norm.
+__device__ __forceinline__ double project_out(const double* a, double rn, double* b) {
+  double cr = 0.0, ci = 0.0;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    cr = fma(a[2 * j], b[2 * j], fma(a[2 * j + 1], b[2 * j + 1], cr));
+    ci = fma(a[2 * j], b[2 * j + 1], fma(-a[2 * j + 1], b[2 * j], ci));
+  }
+  const double part = fma(cr, cr, ci * ci) * rn;
+  cr *= rn;
+  ci *= rn;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    b[2 * j] = fma(-cr, a[2 * j], fma(ci, a[2 * j + 1], b[2 * j]));
+    b[2 * j + 1] = fma(-cr, a[2 * j + 1], fma(-ci, a[2 * j], b[2 * j + 1]));
+  }
+  return part;
+}
+__device__ __forceinline__ double row_norm2(const double* a) {
+  double n = 0.0;
+#pragma unroll
+  for (int j = 0; j < 6; ++j) n = fma(a[j], a[j], n);
+  return n;
+}
+
+// The same projection with fewer FP64 operations: the FP64 pipe bounds the
+// kernel (90% busy; 2.59 M FP64 matrices: 1,989 us by the definition's sweeps with
+// FP64 atan2 and sincos, which stay for the cases below, 951 here).
+// Row 1 takes a second sweep only where the first took out a sixteenth or more
+// of what it left (in norm squared): else one sweep leaves no more of row 0 than
+// its own rounding, as two do.  Of row 2 only a phase is free: orthonormal to
+// rows 0 and 1 it is e^{i alpha} w, w = conj(r0 x r1), so Gram-Schmidt's two
+// sweeps and normalisation come down to the direction of d = <w, row 2>, and
+// e^{i alpha} = d/|d| is also the determinant.  Dividing by its principal cube
+// root leaves rows 0, 1 times q and w times conj(q)^2, q = e^{-i alpha/3}.  q is
+// formed in FP32 (atan2f, sincosf: the branch of the cube root is that of the
+// signs of d), rounded to multiples of 2^-22 (its square is then exact in FP64)
+// and refined by one step on q^3 d/|d| = 1: with q^3 d/|d| = 1 + z, |z| < 1e-6,
+// q (1 - z/3 + 2/9 z^2) is exact to z^3 < 1e-18.  d/|d| is brought back to the
+// unit circle and q kept in two parts until the rows' norms are in it, as what q
+// rounds by is an error of all rows.  rms error against extended precision and,
+// in brackets, the definition's in FP64: projected matrices rounded to FP32
+// 4.22e-17 (4.31e-17), Gaussian 6.02e-17 (6.34e-17), projected matrices with
+// noise of 1e-3 4.69e-17 (4.48e-17).
+// Returns false where a norm is NaN, zero, or so large or small that it could
+// overflow or underflow here and not in the definition.
 __device__ __forceinline__ bool reunit_fast(double* r) {
   double* a = r;  // rows 0 and 1, not normalised until the end
   double* b = r + 6;
-  double n0 = 0.0;
-#pragma unroll
-  for (int j = 0; j < 6; ++j) n0 = fma(a[j], a[j], n0);
+  const double n0 = row_norm2(a);
   const double inv0 = rsqrt(n0);
   const double rn0 = inv0 * inv0;
-#pragma unroll
-  for (int rep = 0; rep < 2; ++rep) {
-    double cr = 0.0, ci = 0.0;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      cr = fma(a[2 * j], b[2 * j], fma(a[2 * j + 1], b[2 * j + 1], cr));
-      ci = fma(a[2 * j], b[2 * j + 1], fma(-a[2 * j + 1], b[2 * j], ci));
-    }
-    cr *= rn0;
-    ci *= rn0;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      b[2 * j] = fma(-cr, a[2 * j], fma(ci, a[2 * j + 1], b[2 * j]));
-      b[2 * j + 1] = fma(-cr, a[2 * j + 1], fma(-ci, a[2 * j], b[2 * j + 1]));
-    }
+  const double part = project_out(a, rn0, b);
+  double n1 = row_norm2(b);
+  if (part > n1 * 0.0625) {
+    project_out(a, rn0, b);
+    n1 = row_norm2(b);
   }
-  double n1 = 0.0;
-#pragma unroll
-  for (int j = 0; j < 6; ++j) n1 = fma(b[j], b[j], n1);
   const double inv1 = rsqrt(n1);
   // x = a x b; d = sum_j x_j row2_j
   double x[6], dr = 0.0, di = 0.0;
@@ -255,35 +273,35 @@ __device__ __forceinline__ bool reunit_fast(double* r) {
   if (!(n0 > 0x1p-200 && n0 < 0x1p200 && n1 > 0x1p-200 && n1 < 0x1p200 && nd > 0x1p-800 &&
         nd < 0x1p800))
     return false;
-  const double er = dr * invd, ei = di * invd;
+  double er = dr * invd, ei = di * invd;
+  const double ue = -0.5 * fma(er, er, fma(ei, ei, -1.0));
+  er = fma(er, ue, er);
+  ei = fma(ei, ue, ei);
   float qs, qc;
   sincosf(atan2f(__double2float_rn(ei), __double2float_rn(er)) * (-1.0f / 3.0f), &qs, &qc);
-  const double tr = (double)qc, ti = (double)qs;
-  double sr, si, zr, zi;
-  zmul(sr, si, tr, ti, tr, ti);
+  const double tr = (double)__fsub_rn(__fadd_rn(qc, 3.0f), 3.0f);
+  const double ti = (double)__fsub_rn(__fadd_rn(qs, 3.0f), 3.0f);
+  double sr = fma(tr, tr, -(ti * ti)), si = (tr + tr) * ti, zr, zi;
   zmul(zr, zi, sr, si, tr, ti);
   sr = fma(zr, er, fma(-zi, ei, -1.0));
   si = fma(zr, ei, zi * er);
   // 1 - z/3 + 2/9 z^2 = 1 + z (2/9 z - 1/3)
   zmul(zr, zi, sr, si, fma(sr, 2.0 / 9.0, -1.0 / 3.0), si * (2.0 / 9.0));
-  const double qr = fma(tr, zr, fma(-ti, zi, tr)), qi = fma(tr, zi, fma(ti, zr, ti));
-  // rows 0, 1: q times the normalised rows; row 2: e^{i alpha} q conj(x) / |x|,
-  // the conjugate of x times conj(e^{i alpha} q) / |x|
-  double n2 = 0.0;
-#pragma unroll
-  for (int j = 0; j < 6; ++j) n2 = fma(x[j], x[j], n2);
-  const double inv2 = rsqrt(n2);
+  const double hr = fma(tr, zr, -(ti * zi)), hi = fma(tr, zi, ti * zr);  // q = t + h
+  const double qr = tr + hr, qi = ti + hi;
+  // rows 0, 1: q over the norms, times the rows; row 2: e^{i alpha} q conj(x) /
+  // |x|, the conjugate of x/|x| times conj(e^{i alpha} q) (its norm taken with q
+  // as for rows 0, 1 costs 0.2e-17 of row 2's error)
+  const double inv2 = rsqrt(row_norm2(x));
   const double pr = fma(er, qr, -(ei * qi)), pi = -fma(er, qi, ei * qr);
+  const double q0r = fma(tr, inv0, hr * inv0), q0i = fma(ti, inv0, hi * inv0);
+  const double q1r = fma(tr, inv1, hr * inv1), q1i = fma(ti, inv1, hi * inv1);
 #pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    a[j] *= inv0;
-    b[j] *= inv1;
-    x[j] *= inv2;
-  }
+  for (int j = 0; j < 6; ++j) x[j] *= inv2;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    zmul(r[2 * j], r[2 * j + 1], a[2 * j], a[2 * j + 1], qr, qi);
-    zmul(r[6 + 2 * j], r[6 + 2 * j + 1], b[2 * j], b[2 * j + 1], qr, qi);
+    zmul(r[2 * j], r[2 * j + 1], a[2 * j], a[2 * j + 1], q0r, q0i);
+    zmul(r[6 + 2 * j], r[6 + 2 * j + 1], b[2 * j], b[2 * j + 1], q1r, q1i);
     zmul(r[12 + 2 * j], r[12 + 2 * j + 1], x[2 * j], x[2 * j + 1], pr, pi);
     r[12 + 2 * j + 1] = -r[12 + 2 * j + 1];
   }

@@ -88,3 +88,27 @@ def test_projection_at_the_edges_of_the_fast_path(su3s):
     assert np.array_equal(np.isnan(got).any((1, 2, 3)), np.isnan(ref).any((1, 2, 3)))
     fine = ~np.isnan(ref).any((1, 2, 3))
     assert np.abs(got - ref)[fine].max() < 1e-14
+
+
+@pytest.mark.parametrize("ratio", [0.0, 0.24, 0.2499, 0.2501, 0.26, 1.0, 1e3, 1e6])
+def test_projection_with_rows_near_each_other(su3s, ratio):
+    """Row 1 = ratio (a phase of row 0) + a unit row orthogonal to it, around the part from which a
+    second sweep is taken (a quarter in norm) and far past it: special unitary to rounding, and the
+    rows of the definition to the rounding of the input, which the ratio magnifies."""
+    rng = np.random.default_rng(23)
+    n = 700
+    q = np.linalg.qr(rng.standard_normal((n, 3, 3)) + 1j * rng.standard_normal((n, 3, 3)))[0]
+    ph = np.exp(2j * np.pi * rng.random((n, 1)))
+    m = np.stack([3.0 * q[:, :, 0], 0.5 * (q[:, :, 1] + ratio * ph * q[:, :, 0]),
+                  q[:, :, 2] + 0.3 * q[:, :, 0] - 0.2j * q[:, :, 1]], 1)
+    x = np.stack([m.real, m.imag], -1)
+    f = su3s.Field(su3s.Lattice((n, 1, 1, 1)))
+    f.upload(x)
+    su3s.reunitarize(f, f)
+    got = f.download()
+    u = got[..., 0] + 1j * got[..., 1]
+    # 2^-53 times: norms and products of 3 complex terms (16), the phase (8), twice for two rows
+    eps = 2.0 ** -53 * 48
+    assert np.abs(u @ np.conj(np.swapaxes(u, 1, 2)) - np.eye(3)).max() < eps
+    assert np.abs(np.linalg.det(u) - 1).max() < 2 * eps
+    assert np.abs(got - oracle.reunitarize(x)).max() < eps * (1 + ratio)
