@@ -145,13 +145,15 @@ __global__ void __launch_bounds__(256) k_batch_tma(const BItem* __restrict__ ite
     if (in < end)
       issue_tile<Tree, P_F64, false>(lane, items[Tn.item].k, nullptr, nullptr, Tn.s0, Tn.mu, buf, bar);
 #pragma unroll
-    for (int k = 0; k < (NS > 0 ? NS : 1); ++k) ctx.sc[k] = M::scalar(p.sc[k], p.sch[k], p.scl[k]);
+    for (int k = 0; k < (NS > 0 ? NS : 1); ++k)
+      ctx.sc[k] = root_scalar<Tree, M>(p.sc[k], p.sch[k], p.scl[k], k);
     if (M::kGuard && __any_sync(0xffffffffu, guard_trips<Tree>(ctx.gmax))) {
       eval_site_f64<Tree, P_F64>(p, T.s0 + lane, T.mu);
     } else {
-      typename M::A acc[1][W];
-      acc_into<Tree, M, true, 1>(ctx, acc[0]);
-      store_obj<Tree::kind, P_F64, M, 1, W>(p.dst, T.s0 + lane, T.mu, acc);
+      using RM = typename RootMath<Tree, M>::type;
+      typename RM::A acc[1][W];
+      root_into<Tree, M>(ctx, acc[0]);
+      store_obj<Tree::kind, P_F64, RM, 1, W>(p.dst, T.s0 + lane, T.mu, acc);
     }
     T = Tn;
     i = in;

@@ -92,7 +92,7 @@ __device__ __forceinline__ void rebuild_row2(typename M::R* m) {
 }
 
 // Load leaf slot I (kind K) of VPS consecutive sites starting at site s.
-template <int K, int PREC, class M, int VPS, class C>
+template <int K, int PREC, class M, int VPS, bool RAW = false, class C>
 __device__ __forceinline__ void load_obj(const FieldDesc& f, int64_t s, int mu, C* ctx, int slot) {
   const int64_t b = elem_base(f, s, mu);
   if constexpr (K == KR) {
@@ -128,7 +128,7 @@ __device__ __forceinline__ void load_obj(const FieldDesc& f, int64_t s, int mu, 
       }
     }
     if constexpr (M::kGuard) ctx[0].gmax = max(ctx[0].gmax, guard_reduce<NC>(gm));
-    if constexpr (PREC == P_F64 || PREC == P_F64_C12) {
+    if constexpr (!RAW && (PREC == P_F64 || PREC == P_F64_C12)) {
 #pragma unroll
       for (int v = 0; v < VPS; ++v) M::template normalize_obj<2 * NC>(ctx[v].leaf[slot]);
     }
@@ -139,13 +139,13 @@ __device__ __forceinline__ void load_obj(const FieldDesc& f, int64_t s, int mu, 
   }
 }
 
-template <class Tree, int I, int PREC, class M, int VPS, class C>
+template <class Tree, int I, int PREC, class M, int VPS, bool GRAD = false, class C>
 __device__ __forceinline__ void load_leaves(const KParams& p, int64_t s, int mu, C* ctx) {
   if constexpr (I < Tree::nleaf) {
     constexpr int K = LeafKind<Tree, I>::value;
     static_assert(K >= 0, "leaf slots must be numbered densely");
-    load_obj<K, PREC, M, VPS>(p.leaf[I], s, mu, ctx, I);
-    load_leaves<Tree, I + 1, PREC, M, VPS>(p, s, mu, ctx);
+    load_obj<K, PREC, M, VPS, !GRAD && LinearTail<Tree, M>::slot == I>(p.leaf[I], s, mu, ctx, I);
+    load_leaves<Tree, I + 1, PREC, M, VPS, GRAD>(p, s, mu, ctx);
   }
 }
 
@@ -199,7 +199,7 @@ __device__ __forceinline__ void eval_sites(const KParams& p, int64_t t, int mu) 
   for (int v = 0; v < VPS; ++v) {
 #pragma unroll
     for (int k = 0; k < (NS > 0 ? NS : 1); ++k)
-      ctx[v].sc[k] = M::scalar(p.sc[k], p.sch[k], p.scl[k]);
+      ctx[v].sc[k] = root_scalar<Tree, M>(p.sc[k], p.sch[k], p.scl[k], k);
     ctx[v].gmax = p.gscal;
   }
   const int64_t s = t * VPS;
@@ -210,19 +210,11 @@ __device__ __forceinline__ void eval_sites(const KParams& p, int64_t t, int mu) 
       return;
     }
   }
-  typename M::A acc[VPS][W];
+  using RM = typename RootMath<Tree, M>::type;
+  typename RM::A acc[VPS][W];
 #pragma unroll
-  for (int v = 0; v < VPS; ++v) {
-    if constexpr (Tree::accumulates) {
-      acc_into<Tree, M, true, 1>(ctx[v], acc[v]);
-    } else {
-      typename M::R val[W];
-      value<Tree, M>(ctx[v], val);
-#pragma unroll
-      for (int r = 0; r < W; ++r) acc[v][r] = M::to_acc(val[r]);
-    }
-  }
-  store_obj<Tree::kind, PREC, M, VPS, W>(p.dst, s, mu, acc);
+  for (int v = 0; v < VPS; ++v) root_into<Tree, M>(ctx[v], acc[v]);
+  store_obj<Tree::kind, PREC, RM, VPS, W>(p.dst, s, mu, acc);
 }
 
 // Evaluation context of one site that loads each leaf from global memory
@@ -371,7 +363,7 @@ __device__ __forceinline__ void adj_site(const GParams& p, int64_t s, int mu) {
   for (int k = 0; k < (NS > 0 ? NS : 1); ++k)
     ctx[0].sc[k] = M::scalar(p.k.sc[k], p.k.sch[k], p.k.scl[k]);
   ctx[0].gmax = p.k.gscal;
-  load_leaves<Tree, 0, P_F64, M, 1>(p.k, s, mu, ctx);
+  load_leaves<Tree, 0, P_F64, M, 1, true>(p.k, s, mu, ctx);
   // dL/dZ
   Ctx<M, 1, 0> g[1];
   load_obj<Tree::kind, P_F64, M, 1>(p.gout, s, mu, g, 0);
@@ -504,7 +496,7 @@ __device__ __forceinline__ void issue_tile(int lane, const KParams& p, const Fie
 }
 
 // Read this lane's site of a staged object into ctx.leaf[slot].
-template <int K, int PREC, class M, class C>
+template <int K, int PREC, class M, bool RAW = false, class C>
 __device__ __forceinline__ void read_obj(const unsigned char* src, int lane, C& ctx, int slot) {
   if constexpr (K == KR) {
     const uint2 v = reinterpret_cast<const uint2*>(src)[lane];
@@ -521,16 +513,17 @@ __device__ __forceinline__ void read_obj(const unsigned char* src, int lane, C& 
       split_complex<M>(v, ctx.leaf[slot][2 * c], ctx.leaf[slot][2 * c + 1]);
     }
     if constexpr (M::kGuard) ctx.gmax = max(ctx.gmax, guard_reduce<NC>(gm));
-    M::template normalize_obj<2 * NC>(ctx.leaf[slot]);
+    if constexpr (!RAW) M::template normalize_obj<2 * NC>(ctx.leaf[slot]);
     if constexpr (K == KM && IsC12<PREC>::value) rebuild_row2<M>(ctx.leaf[slot]);
   }
 }
 
-template <class Tree, int I, int PREC, class M, class C>
+template <class Tree, int I, int PREC, class M, bool GRAD = false, class C>
 __device__ __forceinline__ void read_leaves(const unsigned char* buf, int lane, C& ctx) {
   if constexpr (I < Tree::nleaf) {
-    read_obj<LeafKind<Tree, I>::value, PREC, M>(buf + LeafOff<Tree, PREC, I>::value, lane, ctx, I);
-    read_leaves<Tree, I + 1, PREC, M>(buf, lane, ctx);
+    read_obj<LeafKind<Tree, I>::value, PREC, M, !GRAD && LinearTail<Tree, M>::slot == I>(
+        buf + LeafOff<Tree, PREC, I>::value, lane, ctx, I);
+    read_leaves<Tree, I + 1, PREC, M, GRAD>(buf, lane, ctx);
   }
 }
 
@@ -714,7 +707,8 @@ __device__ __forceinline__ void tma_range(const KParams& p, Units q, unsigned ch
   if (t < ntiles) issue_tile<Tree, PREC, false>(lane, p, nullptr, nullptr, t << 5, mu, buf, bar);
   Ctx<M, NL, NS> ctx;
 #pragma unroll
-  for (int k = 0; k < (NS > 0 ? NS : 1); ++k) ctx.sc[k] = M::scalar(p.sc[k], p.sch[k], p.scl[k]);
+  for (int k = 0; k < (NS > 0 ? NS : 1); ++k)
+    ctx.sc[k] = root_scalar<Tree, M>(p.sc[k], p.sch[k], p.scl[k], k);
   uint32_t phase = 0;
   while (t < ntiles) {
     const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, phase));
@@ -766,16 +760,10 @@ __device__ __forceinline__ void tma_range(const KParams& p, Units q, unsigned ch
     if (M::kGuard && __any_sync(0xffffffffu, guard_trips<Tree>(ctx.gmax))) {
       eval_site_f64<Tree, PREC>(p, (t << 5) + lane, mu);
     } else {
-      typename M::A acc[1][W];
-      if constexpr (Tree::accumulates) {
-        acc_into<Tree, M, true, 1>(ctx, acc[0]);
-      } else {
-        typename M::R val[W];
-        value<Tree, M>(ctx, val);
-#pragma unroll
-        for (int r = 0; r < W; ++r) acc[0][r] = M::to_acc(val[r]);
-      }
-      store_obj<Tree::kind, PREC, M, 1, W>(p.dst, (t << 5) + lane, mu, acc);
+      using RM = typename RootMath<Tree, M>::type;
+      typename RM::A acc[1][W];
+      root_into<Tree, M>(ctx, acc[0]);
+      store_obj<Tree::kind, PREC, RM, 1, W>(p.dst, (t << 5) + lane, mu, acc);
     }
     t = tn;
   }
@@ -843,7 +831,7 @@ __device__ __forceinline__ void adj_tma_range(const GParams& p, Range rg, unsign
     }
     phase ^= 1;
     ctx.gmax = p.k.gscal;
-    read_leaves<Tree, 0, P_F64, M>(buf, lane, ctx);
+    read_leaves<Tree, 0, P_F64, M, true>(buf, lane, ctx);
     Ctx<M, 1, 0> g;
     read_obj<Tree::kind, P_F64, M>(buf + GOFF, lane, g, 0);
     fence_proxy_async_smem();
@@ -973,7 +961,8 @@ struct LazyCtx {
     constexpr int K = I < NL ? LeafKind<Tree, I>::value : Tree::kind;
     wait_leaf<I>();
     Ctx<M, 1, 0> tmp;
-    read_obj<K, PREC, M>(buf + LeafOff<Tree, PREC, I>::value, lane, tmp, 0);
+    read_obj<K, PREC, M, !GRAD && LinearTail<Tree, M>::slot == I>(
+        buf + LeafOff<Tree, PREC, I>::value, lane, tmp, 0);
     if constexpr (M::kGuard) gmax = max(gmax, tmp.gmax);
 #pragma unroll
     for (int r = 0; r < W; ++r) out[r] = tmp.leaf[0][r];
@@ -1039,7 +1028,8 @@ __device__ __forceinline__ void lazy_setup(LazyCtx<Tree, M, PREC, GRAD>& c, unsi
   __syncwarp();
 #pragma unroll
   for (int k = 0; k < (Tree::nsc > 0 ? Tree::nsc : 1); ++k)
-    c.sc[k] = M::scalar(p.sc[k], p.sch[k], p.scl[k]);
+    c.sc[k] = GRAD ? M::scalar(p.sc[k], p.sch[k], p.scl[k])
+                   : root_scalar<Tree, M>(p.sc[k], p.sch[k], p.scl[k], k);
 }
 
 template <class Tree, class M, int PREC>
@@ -1056,20 +1046,14 @@ __device__ __forceinline__ void lazy_range(const KParams& p, Range rg, unsigned 
     c.has_next = tn < ntiles;
     c.next_s0 = tn << 5;
     c.gmax = p.gscal;
-    typename M::A acc[1][W];
-    if constexpr (Tree::accumulates) {
-      acc_into<Tree, M, true, 1>(c, acc[0]);
-    } else {
-      typename M::R val[W];
-      value<Tree, M>(c, val);
-#pragma unroll
-      for (int r = 0; r < W; ++r) acc[0][r] = M::to_acc(val[r]);
-    }
+    using RM = typename RootMath<Tree, M>::type;
+    typename RM::A acc[1][W];
+    root_into<Tree, M>(c, acc[0]);
     c.template refill_repeated<0>();
     if (c.dead) break;
     if (M::kGuard && __any_sync(0xffffffffu, guard_trips<Tree>(c.gmax)))
       eval_site_f64<Tree, PREC>(p, (t << 5) + c.lane, c.mu);
-    else store_obj<Tree::kind, PREC, M, 1, W>(p.dst, (t << 5) + c.lane, c.mu, acc);
+    else store_obj<Tree::kind, PREC, RM, 1, W>(p.dst, (t << 5) + c.lane, c.mu, acc);
     c.parity ^= 1;
     t = tn;
   }
@@ -1330,7 +1314,7 @@ struct RingCtx {
     }
     ph ^= 1u << b;
     Ctx<M, 1, 0> tmp;
-    read_obj<K, PREC, M>(buf + b * L::BUF, lane, tmp, 0);
+    read_obj<K, PREC, M, !GRAD && LinearTail<Tree, M>::slot == I>(buf + b * L::BUF, lane, tmp, 0);
     if constexpr (M::kGuard) gmax = max(gmax, tmp.gmax);
 #pragma unroll
     for (int r = 0; r < W; ++r) out[r] = tmp.leaf[0][r];
@@ -1381,7 +1365,8 @@ __device__ __forceinline__ void ring_setup(RingCtx<Tree, M, PREC, GRAD>& c, unsi
   __syncwarp();
 #pragma unroll
   for (int k = 0; k < (Tree::nsc > 0 ? Tree::nsc : 1); ++k)
-    c.sc[k] = M::scalar(p.sc[k], p.sch[k], p.scl[k]);
+    c.sc[k] = GRAD ? M::scalar(p.sc[k], p.sch[k], p.scl[k])
+                   : root_scalar<Tree, M>(p.sc[k], p.sch[k], p.scl[k], k);
 }
 
 template <class Tree, class M, int PREC>
@@ -1398,19 +1383,13 @@ __device__ __forceinline__ void ring_range(const KParams& p, Range rg, unsigned 
     c.has_next = tn < ntiles;
     c.next_s0 = tn << 5;
     c.gmax = p.gscal;
-    typename M::A acc[1][W];
-    if constexpr (Tree::accumulates) {
-      acc_into<Tree, M, true, 1>(c, acc[0]);
-    } else {
-      typename M::R val[W];
-      value<Tree, M>(c, val);
-#pragma unroll
-      for (int r = 0; r < W; ++r) acc[0][r] = M::to_acc(val[r]);
-    }
+    using RM = typename RootMath<Tree, M>::type;
+    typename RM::A acc[1][W];
+    root_into<Tree, M>(c, acc[0]);
     if (c.dead) break;
     if (M::kGuard && __any_sync(0xffffffffu, guard_trips<Tree>(c.gmax)))
       eval_site_f64<Tree, PREC>(p, (t << 5) + c.lane, c.mu);
-    else store_obj<Tree::kind, PREC, M, 1, W>(p.dst, (t << 5) + c.lane, c.mu, acc);
+    else store_obj<Tree::kind, PREC, RM, 1, W>(p.dst, (t << 5) + c.lane, c.mu, acc);
     t = tn;
   }
   if (c.dead) c.drain();
