@@ -76,7 +76,10 @@ struct BWTile {
 // its descriptors stay in L1) and walks it with the whole-tile TMA pipeline of
 // the single-lattice kernels: one tensor copy per object, the next tile's
 // copies in flight while the current one is computed.  Tensor maps and
-// descriptors are read from the item table in global memory.
+// descriptors are read from the item table in global memory.  Tiles strided by
+// all warps, as in the single-lattice kernels, change item almost every tile and
+// were slower for sums (64 lattices of about 16^4: 606 us against 576), runs of
+// 2 to 32 tiles too (605-691).
 template <class M, class Tree>
 __global__ void __launch_bounds__(256) k_batch_tma(const BItem* __restrict__ items,
                                                    const BWTile* __restrict__ wt, int64_t n,
@@ -109,14 +112,23 @@ __global__ void __launch_bounds__(256) k_batch_tma(const BItem* __restrict__ ite
   while (i < end) {
     const int64_t in = i + 1;
     const BWTile Tn = in < end ? wt[in] : T;   // read while this tile's copies land
+    // The item's parameters while the copies land: read after the wait, their
+    // latency stands between the arrival and the stores.  64 lattices of about
+    // 16^4: a*b 375 -> 331 us, a*b + c*d 590 -> 574, a*b*c + s*d 630 -> 605,
+    // commutator 529 -> 495.
     const KParams& p = items[T.item].k;
+    const FieldDesc dst = p.dst;
+    const uint32_t gscal = p.gscal;
+#pragma unroll
+    for (int k = 0; k < (NS > 0 ? NS : 1); ++k)
+      ctx.sc[k] = root_scalar<Tree, M>(p.sc[k], p.sch[k], p.scl[k], k);
     const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, phase));
     if (!ok) {
       if (lane == 0) report_timeout(err, bar, phase);
       break;
     }
     phase ^= 1;
-    ctx.gmax = p.gscal;
+    ctx.gmax = gscal;
     if constexpr (TwoProducts<Tree>::value) {
       // the first product's leaves, the product, then the second's (as the
       // whole-tile single-lattice kernel)
@@ -133,7 +145,7 @@ __global__ void __launch_bounds__(256) k_batch_tma(const BItem* __restrict__ ite
         eval_site_f64<Tree, P_F64>(p, T.s0 + lane, T.mu);
       } else {
         mul_combine<M, TP::S1>(ctx, acc[0], (typename TP::P1*)nullptr);
-        store_obj<Tree::kind, P_F64, M, 1, W>(p.dst, T.s0 + lane, T.mu, acc);
+        store_obj<Tree::kind, P_F64, M, 1, W>(dst, T.s0 + lane, T.mu, acc);
       }
       T = Tn;
       i = in;
@@ -144,16 +156,13 @@ __global__ void __launch_bounds__(256) k_batch_tma(const BItem* __restrict__ ite
     __syncwarp();
     if (in < end)
       issue_tile<Tree, P_F64, false>(lane, items[Tn.item].k, nullptr, nullptr, Tn.s0, Tn.mu, buf, bar);
-#pragma unroll
-    for (int k = 0; k < (NS > 0 ? NS : 1); ++k)
-      ctx.sc[k] = root_scalar<Tree, M>(p.sc[k], p.sch[k], p.scl[k], k);
     if (M::kGuard && __any_sync(0xffffffffu, guard_trips<Tree>(ctx.gmax))) {
       eval_site_f64<Tree, P_F64>(p, T.s0 + lane, T.mu);
     } else {
       using RM = typename RootMath<Tree, M>::type;
       typename RM::A acc[1][W];
       root_into<Tree, M>(ctx, acc[0]);
-      store_obj<Tree::kind, P_F64, RM, 1, W>(p.dst, T.s0 + lane, T.mu, acc);
+      store_obj<Tree::kind, P_F64, RM, 1, W>(dst, T.s0 + lane, T.mu, acc);
     }
     T = Tn;
     i = in;
