@@ -132,9 +132,10 @@ __device__ __noinline__ void hop_site_f64(const FieldDesc& dst, const FieldDesc&
   hop_site<MathF64, KIND>(dst, U, v, g, s);
 }
 
-// One thread per site; the grid is one wave, so the sites in flight (and the
-// backward links and neighbours they share) fit the L2 cache, and the loop over
-// the 8 terms is rolled.  Colour matrices: the terms run through a single
+// One thread per site; up to 32 waves of blocks (launch_hop), which start in the
+// order of the sites, so that the sites in flight (and the backward links and
+// neighbours they share) stay together in the L2 cache; the loop over the 8
+// terms is rolled.  Colour matrices: the terms run through a single
 // product routine (the backward link's adjoint is taken in its load), which
 // keeps the matrix-product code small enough for the instruction cache (+29%
 // at 48^4 over separate forward and backward routines).  Colour vectors (native
@@ -310,8 +311,15 @@ static cudaError_t launch_hop(const su3s_field* dest, const su3s_field* U, const
   const LatGeo g = lat_geo(v);
   int per_sm = 1;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hop<M, KIND>, 128, 0);
-  int64_t nb = (int64_t)(per_sm > 0 ? per_sm : 1) * sm_count();   // one wave
+  // 32 waves: the blocks of one wave drift apart over a long grid-stride loop.
+  // 32^3 x 64, one wave, four, 32: pair arithmetic on matrices 1,086, 998, 955 us;
+  // fixed point on vectors 604, 548, 536, on matrices 1,361, 1,358, 1,345; FP64
+  // 1,212, 1,177, 1,175 and 3,700, 3,602, 3,579.  Fixed-point matrices below eight
+  // waves keep one: 94.8 us against 96.8 at 16^3 x 32, 3.4 waves (230 against
+  // 228 at 8.5).
+  const int64_t wave = (int64_t)(per_sm > 0 ? per_sm : 1) * sm_count();
   const int64_t need = (g.V + 127) / 128;
+  const int64_t nb = M::kScaled && KIND == KM && need < 8 * wave ? wave : 32 * wave;
   const dim3 grid((unsigned)(nb < need ? nb : need));
   k_hop<M, KIND><<<grid, 128, 0, st>>>(dest->desc, U->desc, v->desc, g);
   return cudaGetLastError();

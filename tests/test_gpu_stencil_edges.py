@@ -3,6 +3,7 @@ computed in native FP64 then, so it equals that arithmetic's kernel), blocks wit
 extents of 1 and 2 (a site that is its own neighbour), and mixed layouts of the fields."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import synth
@@ -100,3 +101,50 @@ def test_vector_hop_ragged_blocks_and_mixed_layouts(su3s, dims):
     z = su3s.Field(lat, su3s.VECTOR, 1, su3s.F64, su3s.AOSOA, 4)
     su3s.hop(z, U, X)
     assert np.abs(z.download() - oracle.hop(u, x, dims)).max() < 8e-13
+
+
+@pytest.mark.parametrize("dims", [(16, 16, 16, 32), (17, 16, 32, 48), (96, 64, 32, 33)])
+@pytest.mark.parametrize("math", ["MATH_F64", "MATH_DF32", "MATH_FX"])
+def test_neighbour_terms_over_the_waves_of_a_launch(su3s, dims, math):
+    """One wave of blocks, several, and more sites than 32 waves take (threads then take several):
+    the hopping terms on vectors and matrices at sites spread over the lattice against their sums in
+    FP64, and the Wilson term on every site against another arithmetic's launch."""
+    lat = su3s.Lattice(dims)
+    g = torch.Generator(device="cuda").manual_seed(29)
+    fill = lambda f: f.tensor.copy_(torch.rand(f.tensor.shape, dtype=torch.float64, device="cuda", generator=g) - 0.5)
+    U = su3s.Field(lat, su3s.MATRIX, 4)
+    fill(U)
+    lx, ly, lz, lt = dims
+    V = lx * ly * lz * lt
+    rng = np.random.default_rng(5)
+    sites = np.unique(np.r_[0, V - 1, V // 2, rng.integers(0, V, 200)])
+    crd = np.stack([sites % lx, sites // lx % ly, sites // (lx * ly) % lz, sites // (lx * ly * lz)], 1)
+
+    def at(field, index, mu=0):   # (n, rows, cols) complex of a structure-of-arrays field
+        nc = {su3s.MATRIX: 9, su3s.VECTOR: 3}[field.kind]
+        t = field.tensor.view(field.nmu * nc, -1, 2)[mu * nc:(mu + 1) * nc, torch.as_tensor(index, device="cuda")]
+        return torch.view_as_complex(t.contiguous()).T.cpu().numpy().reshape(len(index), 3, nc // 3)
+
+    def neighbour(mu, sign):
+        c = crd.copy()
+        c[:, mu] = (c[:, mu] + sign) % dims[mu]
+        return c[:, 0] + lx * (c[:, 1] + ly * (c[:, 2] + lz * c[:, 3]))
+
+    for kind in (su3s.VECTOR, su3s.MATRIX):
+        v = su3s.Field(lat, kind)
+        fill(v)
+        z = v.like()
+        su3s.hop(z, U, v, getattr(su3s, math))
+        ref = 0
+        for mu in range(4):
+            n, p = neighbour(mu, 1), neighbour(mu, -1)
+            ref = ref + at(U, sites, mu) @ at(v, n) + np.conj(np.swapaxes(at(U, p, mu), 1, 2)) @ at(v, p)
+        # 5.7e-14 is the pair arithmetic's error for 6 real products of unit size; here 48 below 1/4
+        assert np.abs(at(z, sites) - ref).max() < 1.2e-13
+    # the Wilson term (48 real products below 1/2) against native FP64's launch
+    psi = su3s.Field(lat, su3s.VECTOR, 4)
+    fill(psi)
+    z, w = psi.like(), psi.like()
+    su3s.dslash(z, U, psi, getattr(su3s, math))
+    su3s.dslash(w, U, psi, su3s.MATH_DF32 if math == "MATH_F64" else su3s.MATH_F64)
+    assert ((z.tensor - w.tensor).view(12, -1, 2)[:, :V].abs().max() < 2.4e-13).item()
