@@ -682,17 +682,18 @@ __device__ __forceinline__ void acc_node(const C& ctx, typename M::A* acc, Scale
   vec_scale_add<M, W, FIRST, SG>(acc, ctx.sc[K], v);
 }
 
-// Products plus or minus a term linear in a leaf, X Y + s z (a*b*c + s*d), in
-// the fixed-point arithmetic: the product alone is evaluated in it, and s z is
+// Products plus or minus a term linear in a leaf, X Y + s z (a*b*c + s*d): the
+// product alone is evaluated in the pair or fixed-point arithmetic, and s z is
 // added to the converted result in FP64, one fused multiply-add per real on a
-// pipe that is otherwise idle.  In fixed point the term costs about 45 integer
-// operations per real (the leaf's alignment to its largest element, the scaled
-// product, two 64-bit shifts to a common scale).  The leaf enters exactly
-// instead of cut to its largest element's last bit, and the result is rounded
-// once more: a*b*c + 0.5*d 7.6e-16 -> 7.3e-16 at most against extended precision.
-// Measured at 32^4 in blocks of 64 sites: 195 -> 169 us; 20^4 32.1 -> 32.0, 48^4
-// 965 -> 830.  Sums without a product keep the fixed point: their conversions
-// and additions alone would fill the FP64 pipe (s*a + b on 24^4 23 -> 29 us).
+// pipe that is otherwise idle.  In pairs the term costs the leaf's split and five
+// packed operations per real, in fixed point about 45 integer operations (the
+// leaf's alignment to its largest element, the scaled product, two 64-bit shifts
+// to a common scale).  The leaf enters exactly, and the result is rounded once
+// more (fixed point: 7.6e-16 -> 7.3e-16 at most against 64 bits).
+// Measured, whole-tile staging, SoA: pairs 20^4 26.2 -> 23.5 us, 32^4 133 -> 116, 48^4
+// 618 -> 544 (7.0 TB/s); fixed point 20^4 32.1 -> 32.0, 32^4 195 -> 169, 48^4 965 -> 819.
+// Sums without a product stay as they are: their conversions and additions alone
+// would fill the FP64 pipe (s*a + b in fixed point on 24^4: 23 -> 29 us).
 template <class Tree, class M>
 struct LinearTail {
   static constexpr bool value = false;
@@ -721,7 +722,7 @@ struct LinearTailOf {
   using Term = TailTerm<Y>;
   static constexpr int sign = SG;
   static constexpr bool value =
-      M::kScaled && IsMulNode<X>::value && Term::value && Count<X, Term::slot>::value == 0;
+      (M::kScaled || M::kPaired) && IsMulNode<X>::value && Term::value && Count<X, Term::slot>::value == 0;
   static constexpr int slot = value ? Term::slot : -1;
 };
 template <class X, class Y, class M>
@@ -745,30 +746,39 @@ __device__ __forceinline__ typename M::R root_scalar(double s, float sh, float s
   if constexpr (LinearTail<Tree, M>::value) {
     using T = typename LinearTail<Tree, M>::Term;
     if (T::scaled && k == T::k)
-      return M::from_bits((uint32_t)__double2loint(s), (uint32_t)__double2hiint(s));
+      return raw_bits<M>((uint32_t)__double2loint(s), (uint32_t)__double2hiint(s));
   }
   return M::scalar(s, sh, sl);
 }
 
-// The tree's result (a linear last term's leaf and factor are FP64 bits).
+// The product of a tree with a linear last term, in FP64, and the term added to
+// it (y: the leaf's FP64 bits; its factor is held as bits too).
+template <class Tree, class M, class C>
+__device__ __forceinline__ void root_product(const C& ctx, double* acc) {
+  constexpr int W = Width<Tree::kind>::value;
+  typename M::A a[W];
+  acc_into<typename LinearTail<Tree, M>::Head, M, true, 1>(ctx, a);
+#pragma unroll
+  for (int r = 0; r < W; r += 2) complex_to_f64<M>(a[r], a[r + 1], acc[r], acc[r + 1]);
+}
+template <class Tree, class M, class C>
+__device__ __forceinline__ void root_add(const C& ctx, const typename M::R* y, double* acc) {
+  using T = LinearTail<Tree, M>;
+  double s = T::sign;
+  if constexpr (T::Term::scaled) s *= raw_value<M>(ctx.sc[T::Term::k]);
+#pragma unroll
+  for (int r = 0; r < Width<Tree::kind>::value; ++r) acc[r] = fma(s, raw_value<M>(y[r]), acc[r]);
+}
+
+// The tree's result.
 template <class Tree, class M, class C>
 __device__ __forceinline__ void root_into(const C& ctx, typename RootMath<Tree, M>::type::A* acc) {
   constexpr int W = Width<Tree::kind>::value;
   if constexpr (LinearTail<Tree, M>::value) {
-    using T = LinearTail<Tree, M>;
-    typename M::A a[W];
-    acc_into<typename T::Head, M, true, 1>(ctx, a);
-#pragma unroll
-    for (int r = 0; r < W; ++r) acc[r] = M::to_f64(a[r]);
-    double s = T::sign;
-    if constexpr (T::Term::scaled) {
-      const typename M::R f = ctx.sc[T::Term::k];
-      s *= __hiloint2double(f.h, f.l);
-    }
+    root_product<Tree, M>(ctx, acc);
     typename M::R y[W];
-    ctx.template leaf_value<T::slot, W>(y);
-#pragma unroll
-    for (int r = 0; r < W; ++r) acc[r] = fma(s, __hiloint2double(y[r].h, y[r].l), acc[r]);
+    ctx.template leaf_value<LinearTail<Tree, M>::slot, W>(y);
+    root_add<Tree, M>(ctx, y, acc);
   } else if constexpr (Tree::accumulates) {
     acc_into<Tree, M, true, 1>(ctx, acc);
   } else {

@@ -91,7 +91,8 @@ __device__ __forceinline__ void rebuild_row2(typename M::R* m) {
   if constexpr (M::kScaled) M::template finish_obj<18>(m, a);
 }
 
-// Load leaf slot I (kind K) of VPS consecutive sites starting at site s.
+// Load leaf slot I (kind K) of VPS consecutive sites starting at site s (RAW: as
+// its FP64 bits, for a linear last term).
 template <int K, int PREC, class M, int VPS, bool RAW = false, class C>
 __device__ __forceinline__ void load_obj(const FieldDesc& f, int64_t s, int mu, C* ctx, int slot) {
   const int64_t b = elem_base(f, s, mu);
@@ -117,7 +118,12 @@ __device__ __forceinline__ void load_obj(const FieldDesc& f, int64_t s, int mu, 
         static_assert(VPS == 1, "guarded arithmetics read FP64 storage");
         const uint4 v = ld16((const char*)f.ptr + (b + c * f.s_c) * 16);
         gm[c] = guard_max(0u, v.y, v.w);
-        split_complex<M>(v, re[0], im[0]);
+        if constexpr (RAW) {
+          re[0] = raw_bits<M>(v.x, v.y);
+          im[0] = raw_bits<M>(v.z, v.w);
+        } else {
+          split_complex<M>(v, re[0], im[0]);
+        }
       } else {
         St::template load<M>(f.ptr, b + c * f.s_c, re, im);
       }
@@ -139,12 +145,24 @@ __device__ __forceinline__ void load_obj(const FieldDesc& f, int64_t s, int mu, 
   }
 }
 
+// Plain loads: a linear last term's leaf is read after the product in the pair
+// arithmetic, where its registers are free by then ((a*b)*c + s*d at 48^4: 959 us
+// with the term in pairs, 1,111 with the leaf read first, 941 after); in fixed
+// point it is read first (32^4: 198 us against 214).
+template <class Tree, class M>
+struct LateTail {
+  static constexpr bool value = LinearTail<Tree, M>::value && M::kPaired;
+};
+
 template <class Tree, int I, int PREC, class M, int VPS, bool GRAD = false, class C>
 __device__ __forceinline__ void load_leaves(const KParams& p, int64_t s, int mu, C* ctx) {
   if constexpr (I < Tree::nleaf) {
     constexpr int K = LeafKind<Tree, I>::value;
     static_assert(K >= 0, "leaf slots must be numbered densely");
-    load_obj<K, PREC, M, VPS, !GRAD && LinearTail<Tree, M>::slot == I>(p.leaf[I], s, mu, ctx, I);
+    if constexpr (GRAD || LinearTail<Tree, M>::slot != I)
+      load_obj<K, PREC, M, VPS>(p.leaf[I], s, mu, ctx, I);
+    else if constexpr (!LateTail<Tree, M>::value)
+      load_obj<K, PREC, M, VPS, true>(p.leaf[I], s, mu, ctx, I);
     load_leaves<Tree, I + 1, PREC, M, VPS, GRAD>(p, s, mu, ctx);
   }
 }
@@ -212,8 +230,20 @@ __device__ __forceinline__ void eval_sites(const KParams& p, int64_t t, int mu) 
   }
   using RM = typename RootMath<Tree, M>::type;
   typename RM::A acc[VPS][W];
+  if constexpr (LateTail<Tree, M>::value) {
+    root_product<Tree, M>(ctx[0], acc[0]);
+    constexpr int I = LinearTail<Tree, M>::slot;
+    Ctx<M, 1, 0> y[1];
+    load_obj<LeafKind<Tree, I>::value, PREC, M, 1, true>(p.leaf[I], s, mu, y, 0);
+    if (M::kGuard && guard_trips<Tree>(y[0].gmax)) {
+      eval_site_f64<Tree, PREC>(p, s, mu);
+      return;
+    }
+    root_add<Tree, M>(ctx[0], y[0].leaf[0], acc[0]);
+  } else {
 #pragma unroll
-  for (int v = 0; v < VPS; ++v) root_into<Tree, M>(ctx[v], acc[v]);
+    for (int v = 0; v < VPS; ++v) root_into<Tree, M>(ctx[v], acc[v]);
+  }
   store_obj<Tree::kind, PREC, RM, VPS, W>(p.dst, s, mu, acc);
 }
 
@@ -495,7 +525,7 @@ __device__ __forceinline__ void issue_tile(int lane, const KParams& p, const Fie
   __syncwarp();
 }
 
-// Read this lane's site of a staged object into ctx.leaf[slot].
+// Read this lane's site of a staged object into ctx.leaf[slot] (RAW: its bits).
 template <int K, int PREC, class M, bool RAW = false, class C>
 __device__ __forceinline__ void read_obj(const unsigned char* src, int lane, C& ctx, int slot) {
   if constexpr (K == KR) {
@@ -510,7 +540,12 @@ __device__ __forceinline__ void read_obj(const unsigned char* src, int lane, C& 
     for (int c = 0; c < NC; ++c) {
       const uint4 v = reinterpret_cast<const uint4*>(src + c * 512)[lane];
       if constexpr (M::kGuard) gm[c] = guard_max(0u, v.y, v.w);
-      split_complex<M>(v, ctx.leaf[slot][2 * c], ctx.leaf[slot][2 * c + 1]);
+      if constexpr (RAW) {
+        ctx.leaf[slot][2 * c] = raw_bits<M>(v.x, v.y);
+        ctx.leaf[slot][2 * c + 1] = raw_bits<M>(v.z, v.w);
+      } else {
+        split_complex<M>(v, ctx.leaf[slot][2 * c], ctx.leaf[slot][2 * c + 1]);
+      }
     }
     if constexpr (M::kGuard) ctx.gmax = max(ctx.gmax, guard_reduce<NC>(gm));
     if constexpr (!RAW) M::template normalize_obj<2 * NC>(ctx.leaf[slot]);

@@ -791,6 +791,20 @@ __device__ __forceinline__ void split_complex(uint4 v, typename M::R& re, typena
   }
 }
 
+// An FP64 value carried in an operand's registers as its bits, and that value.
+template <class M>
+__device__ __forceinline__ typename M::R raw_bits(uint32_t lo, uint32_t hi) {
+  if constexpr (M::kPaired) return df{__uint_as_float(hi), __uint_as_float(lo)};
+  else return M::from_bits(lo, hi);
+}
+template <class M>
+__device__ __forceinline__ double raw_value(const typename M::R& x) {
+  if constexpr (M::kPaired)
+    return __hiloint2double((int)__float_as_uint(x.h), (int)__float_as_uint(x.l));
+  else
+    return __hiloint2double(x.h, x.l);
+}
+
 // The FP64 values of a complex output's two accumulators (packed for the pair
 // arithmetic, with to_f64's values).
 template <class M>
