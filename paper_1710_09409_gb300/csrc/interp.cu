@@ -16,31 +16,9 @@
 
 #include "dev_kernels.cuh"
 #include "internal.h"
+#include "interp_prog.h"
 
 namespace su3s {
-
-constexpr int kIRegs = 12;
-constexpr int kIMax = 48;
-
-enum IOp : int8_t { I_LOAD = 0, I_MMUL = 1, I_MVMUL = 2, I_RMUL = 3, I_ADD = 4, I_SUB = 5, I_SCALE = 6, I_ADJ = 7 };
-
-struct IIns {
-  int8_t op, dst, a, b;
-  int8_t w;    // width in reals of the result (18, 6, 1)
-  int8_t arg;  // leaf slot (LOAD, with kind in b) / factor index (SCALE)
-  int8_t adj;  // products: 1 the left operand's adjoint, 2 the right one's
-  int8_t pad;
-};
-
-struct IProg {
-  int32_t n;
-  int32_t root;
-  int32_t root_kind;
-  int32_t nregs;   // registers the program uses (shared memory is sized to them)
-  int32_t nloads;  // its loads in order: leaf slot and width in reals
-  int8_t load_leaf[kMaxLeaves], load_w[kMaxLeaves];
-  IIns ins[kIMax];
-};
 
 // The register file: real r of register g of this thread, in a slot of SLOT
 // bytes.  The native FP64 path of the range guard runs on the register file of
@@ -294,8 +272,6 @@ __global__ void __launch_bounds__(128) k_interp(const __grid_constant__ KParams 
 // are slower here (a (b c - d) at 40^4 592 / 561), programs of three products
 // and more too (a b c d at 32^4 228 / 223: their rolled rows keep fewer
 // accumulations in flight), and small lattices, a thread's chain being longer.
-constexpr int64_t kPairSites = 300000;
-constexpr int kPairRegs = 3;
 struct PRegs {
   float4* base;
   int nt, tid;
@@ -566,127 +542,6 @@ __global__ void __launch_bounds__(128) k_interp_pair(const __grid_constant__ KPa
 
 // ------------------------------------------------------------------ host
 namespace {
-struct Builder {
-  IProg prog;
-  bool busy[kIRegs] = {};
-  int leaf_reg[kMaxLeaves];
-  int uses_left[kMaxLeaves] = {};  // leaf nodes of each slot not generated yet
-  const Canon* c;
-  bool reuse = true;  // element-by-element results in place
-  bool fold = true;   // adjoints of a product's operands folded into it
-  int nscal = 0;
-  int err = 0;
-
-  int alloc() {
-    for (int r = 0; r < kIRegs; ++r)
-      if (!busy[r]) {
-        busy[r] = true;
-        if (r + 1 > prog.nregs) prog.nregs = r + 1;
-        return r;
-      }
-    err = 1;
-    return 0;
-  }
-  // whether register r holds a leaf that is still to be used
-  bool kept(int r) const {
-    for (int l = 0; l < kMaxLeaves; ++l)
-      if (leaf_reg[l] == r && uses_left[l] > 0) return true;
-    return false;
-  }
-  // free register r unless it holds a leaf that is still to be used
-  void release(int r) {
-    if (!kept(r)) busy[r] = false;
-  }
-  // register of an element-by-element result: an operand's own if it is not
-  // needed any more (a leaf's register then holds the leaf no longer)
-  int in_place(int a, int b) {
-    const int d = !reuse ? -1 : !kept(a) ? a : !kept(b) ? b : -1;
-    if (d < 0) return alloc();
-    for (int l = 0; l < kMaxLeaves; ++l)
-      if (leaf_reg[l] == d) leaf_reg[l] = -1;
-    return d;
-  }
-  void emit(IIns in) {
-    if (prog.n >= kIMax) {
-      err = 2;
-      return;
-    }
-    prog.ins[prog.n++] = in;
-  }
-  static int8_t width(int kind) { return kind == SU3S_MATRIX ? 18 : kind == SU3S_VECTOR ? 6 : 1; }
-
-  int slot_of(const su3s_field* f) {
-    for (size_t i = 0; i < c->leaves.size(); ++i)
-      if (c->leaves[i] == f) return (int)i;
-    return 0;
-  }
-
-  void count_uses(const su3s_expr* e) {
-    if (e->op == 0) {
-      ++uses_left[slot_of(e->f)];
-      return;
-    }
-    if (e->a) count_uses(e->a);
-    if (e->b) count_uses(e->b);
-  }
-
-  // returns the register holding the node's value
-  int gen(const su3s_expr* e) {
-    if (err) return 0;
-    switch (e->op) {
-      case 0: {  // a leaf: loaded at its first use
-        const int l = slot_of(e->f);
-        if (leaf_reg[l] < 0) {
-          const int r = alloc();
-          leaf_reg[l] = r;
-          const int kind = e->f->kind;
-          emit(IIns{I_LOAD, (int8_t)r, 0, (int8_t)kind, width(kind), (int8_t)l, 0, 0});
-          if (!err) {
-            prog.load_leaf[prog.nloads] = (int8_t)l;
-            prog.load_w[prog.nloads++] = width(kind);
-          }
-        }
-        --uses_left[l];
-        return leaf_reg[l];
-      }
-      case 4: {
-        int k = nscal++;  // factors numbered in the canonical (pre-order) order
-        int a = gen(e->a);
-        int d = in_place(a, a);
-        emit(IIns{I_SCALE, (int8_t)d, (int8_t)a, 0, width(e->kind), (int8_t)k, 0, 0});
-        if (a != d) release(a);
-        return d;
-      }
-      case 5: {
-        int a = gen(e->a);
-        int d = alloc();
-        emit(IIns{I_ADJ, (int8_t)d, (int8_t)a, 0, 18, 0, 0, 0});
-        release(a);
-        return d;
-      }
-      default: {
-        const su3s_expr *ea = e->a, *eb = e->b;
-        int8_t adj = 0, op;
-        if (e->op == 1) {
-          op = e->kind == SU3S_MATRIX ? I_MMUL : e->kind == SU3S_VECTOR ? I_MVMUL : I_RMUL;
-          // a product reads the adjoint of an operand from the operand itself
-          for (; fold && ea->op == 5; ea = ea->a) adj ^= 1;
-          for (; fold && eb->op == 5; eb = eb->a) adj ^= 2;
-        } else {
-          op = e->op == 2 ? I_ADD : I_SUB;
-        }
-        int a = gen(ea);
-        int b = gen(eb);
-        int d = e->op == 1 ? alloc() : in_place(a, b);
-        emit(IIns{op, (int8_t)d, (int8_t)a, (int8_t)b, width(e->kind), 0, adj, 0});
-        if (a != d) release(a);
-        if (b != d) release(b);
-        return d;
-      }
-    }
-  }
-};
-
 template <class M>
 cudaError_t launch_interp(const KParams& p, const IProg& prog, cudaStream_t st) {
   static_assert(!M::kGuard || sizeof(typename M::R) >= sizeof(double),
@@ -767,43 +622,21 @@ static int degree(const su3s_expr* e) {
 }
 
 int interp_eval(const su3s_expr* e, const Canon& c, su3s_field* dest, int math, cudaStream_t st) {
-  // The limits are those of the plain program (one register per result, adjoints
-  // as steps of their own); what runs is never longer.
   // Two sites per thread from kPairSites on, for programs of at most two products
   // whose registers let 8 warps per SM run; else one site per thread.
   const bool large = math == MATH_DF && (int64_t)dest->Vpad * dest->nmu >= kPairSites;
-  Builder bld;
-  int root = 0;
-  bool pairs = false;
-  for (int pass = 0; pass < 3; ++pass) {
-    // 0: the limits; 1: two sites per thread, adjoints read in place; 2: one site
-    if (pass == 1 && !large) continue;
-    bld = Builder();
-    memset(&bld.prog, 0, sizeof bld.prog);
-    bld.c = &c;
-    bld.reuse = pass > 0;
-    bld.fold = pass == 1;
-    for (int l = 0; l < kMaxLeaves; ++l) bld.leaf_reg[l] = -1;
-    bld.count_uses(e);
-    root = bld.gen(e);
-    if (bld.err)
-      return fail(SU3S_EUNSUPPORTED, "expression too large for the interpreter (%d registers, %d steps)",
-                  kIRegs, kIMax);
-    int products = 0;
-    for (int i = 0; i < bld.prog.n; ++i)
-      products += bld.prog.ins[i].op == I_MMUL || bld.prog.ins[i].op == I_MVMUL;
-    pairs = pass == 1 && bld.prog.nregs <= kPairRegs && products <= 2;
-    if (pairs) break;
-  }
-  bld.prog.root = root;
-  bld.prog.root_kind = c.kind;
+  IProg prog;
+  bool pairs;
+  if (interp_program(e, c, large, &prog, &pairs))
+    return fail(SU3S_EUNSUPPORTED, "expression too large for the interpreter (%d registers, %d steps)",
+                kIRegs, kIMax);
   KParams p;
   build_params(c, dest, 1, &p);
   p.ghi = guard_hi(degree(e));
-  cudaError_t ce = math == MATH_F64  ? launch_interp<MathF64>(p, bld.prog, st)
-                   : math == MATH_FX ? launch_interp<MathFX>(p, bld.prog, st)
-                                     : pairs ? launch_interp_pair(p, bld.prog, st)
-                                               : launch_interp<MathDFScalar>(p, bld.prog, st);
+  cudaError_t ce = math == MATH_F64  ? launch_interp<MathF64>(p, prog, st)
+                   : math == MATH_FX ? launch_interp<MathFX>(p, prog, st)
+                                     : pairs ? launch_interp_pair(p, prog, st)
+                                               : launch_interp<MathDFScalar>(p, prog, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "interpreter kernel launch");
   return SU3S_OK;
 }
