@@ -404,21 +404,31 @@ using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t
                                    const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                    CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// The driver's tensor-map encoder, looked up once through the runtime (no
-// link against the driver library); null when no driver is present.
+using CtxGetCurrentFn = CUresult (*)(CUcontext*);
+
+// A driver function, looked up through the runtime (no link against the driver
+// library); null when no driver is present.
+static void* driver_fn(const char* name) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+  if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+      q == cudaDriverEntryPointSuccess)
+    return p;
+  cudaGetLastError();  // clear the lookup's error
+  return nullptr;
+}
+
+// The driver's tensor-map encoder, looked up once, with a context current (it
+// needs one).  A thread that has made no runtime call yet has none: fields made
+// there would have no map and run the plain-load kernels.  A context that the
+// caller has made current stays.
 static EncodeTiledFn encode_tiled() {
-  static EncodeTiledFn fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-    else
-      cudaGetLastError();  // clear the lookup's error
-  });
+  static const auto fn = reinterpret_cast<EncodeTiledFn>(driver_fn("cuTensorMapEncodeTiled"));
+  static const auto current = reinterpret_cast<CtxGetCurrentFn>(driver_fn("cuCtxGetCurrent"));
+  CUcontext ctx = nullptr;
+  int dev = 0;
+  if (fn && current && current(&ctx) == CUDA_SUCCESS && !ctx && cudaGetDevice(&dev) == cudaSuccess)
+    cudaSetDevice(dev);
   return fn;
 }
 
@@ -433,13 +443,6 @@ static void encode_tmap(su3s_field* f) {
   if (f->layout == SU3S_AOSOA && f->block < 32) return;
   EncodeTiledFn enc = encode_tiled();
   if (!enc) return;
-  // The encoder needs a current context.  A thread that has made no runtime call
-  // yet has none (fields made there had no map and ran the plain-load kernels).
-  static thread_local bool have_context = false;
-  if (!have_context) {
-    int dev = 0;
-    have_context = cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess;
-  }
   const uint64_t w = (uint64_t)f->desc.s_c;
   const uint64_t rows = (uint64_t)f->Vpad * f->nmu * f->ncomp / w;
   // tensor-copy coordinates are signed 32-bit: column 2*site (box end 2*w-1)
