@@ -10,11 +10,13 @@ dL/dRe + i dL/dIm.
 """
 import ctypes
 
+import numpy as np
 import torch
 
 from . import F64, MATH_DEFAULT, MATRIX, SOA, _check, _stream, _Tree, load
 
 _OPS = {"mul": 1, "add": 2, "sub": 3}
+_FIXED = (int, float, bool, np.float64)   # number types whose objects never change
 
 
 def _result_kind(tree, kinds):
@@ -35,10 +37,12 @@ class _Program:
     def __init__(self, tree, kinds):
         prog, scalars, self.reads = [], [], set()
         n = len(kinds)
+        given = list(kinds)   # the values the tree is made of
 
         def walk(t):
             op = t[0]
             if op == "leaf":
+                given.append(t[1])
                 i = range(n)[t[1]]
                 self.reads.add(i)
                 prog.extend((0, i))
@@ -47,6 +51,7 @@ class _Program:
                 walk(t[2])
                 prog.extend((_OPS[op], 0))
             elif op == "scale":
+                given.append(t[1])
                 scalars.append(float(t[1]))
                 k = len(scalars) - 1
                 walk(t[2])
@@ -63,8 +68,9 @@ class _Program:
         self.kinds = (ctypes.c_int * n)(*kinds)
         self.kind = _result_kind(tree, kinds)
         self.nprog, self.nscalar, self.nleaf = len(prog) // 2, len(scalars), n
-        # equal keys have equal programs: not so for zeros (0.0 == -0.0)
-        self.keep = all(s != 0.0 for s in scalars)
+        # Equal keys have equal programs, now and later: not so for zeros (0.0 == -0.0), nor for
+        # objects that can change under the same key (a 0-d tensor as a factor, updated in place).
+        self.keep = all(type(x) in _FIXED for x in given) and all(s != 0.0 for s in scalars)
 
 
 _programs = {}
