@@ -1250,9 +1250,7 @@ static cudaError_t launch_split(const SplitAdjoint& sp, int mode, cudaStream_t s
     GParamsSum both;
     both.half[0] = sp.p[0];
     both.half[1] = sp.p[1];
-    // one block per SM in all, an even number for every link
-    int nb = (sm_count() + nmu - 1) / nmu;
-    nb += nb & 1;
+    const int nb = pair_sum_blocks(sm_count(), nmu);
     return e->sum_fn(&both, dim3((unsigned)nb, (unsigned)nmu, 1), dim3(kSumThreads, 1, 1), st);
   }
   cudaError_t ce = launch_planned(sp.ent[0], sp.p[0], sp.tma[0], st);

@@ -95,6 +95,17 @@ int plan_launch(const EvalEntry* e, int64_t nvec, int nmu, bool tma_ok, Launch* 
 bool tma_layout_ok(const su3s_field* f);
 bool tma_tree_ok(const Canon& c, const su3s_field* dest);
 
+// Blocks per link of the reverse mode of two products in one launch: an even
+// number (half for each product), and no more than one block per SM over all
+// links.  A block's buffers take an SM's shared memory, and its share of the
+// units is fixed: what does not fit runs its whole share after the others.
+// Rounded up to an even number (156 blocks for 152 SMs and three links) 24^4 took
+// 386 us, 16^4 73.7; now 217 and 55.9.  Five links 636 and 135, now 357 and 80.
+inline int pair_sum_blocks(int sms, int nmu) {
+  const int nb = (sms / nmu) & ~1;
+  return nb < 2 ? 2 : nb;
+}
+
 // fill a KParams from a canonical tree and destination
 int build_params(const Canon& c, const su3s_field* dest, int vps, KParams* p);
 
