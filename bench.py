@@ -71,8 +71,8 @@ MATH_ERR = {"fx": "7.8e-16 - 1.6e-15",
 # template arguments name it: (tree, arithmetic type, storage, reverse mode).
 # With the data movement the row ran with (the tuner's variant, else the
 # library's default) this gives the kernel ncu names; the reverse mode of
-# a*b+c*d runs split (reported variant 10 + the halves' variant): 14 is both
-# products in one launch, others two launches of the single-product kernel.
+# a*b+c*d runs split: variant 15 is both products in one launch, 10 + the halves'
+# variant two launches of the single-product kernel.
 T_MM = "Mul<LM<0>, LM<1>>"
 T_E1 = "Add<Mul<LM<0>, LM<1>>, Mul<LM<2>, LM<3>>>"
 ROW_TREE = {
@@ -94,7 +94,7 @@ FWD_KERNEL = ["k_eval<{t}, {m}, {p}>", "k_eval_tma<{t}, {m}, {p}>", "k_eval_lazy
 ADJ_KERNEL = ["k_adjoint<{t}, {m}>", "k_adjoint_tma<{t}, {m}>", "k_adjoint_lazy<{t}, {m}>",
               "k_adjoint_ring<{t}, {m}>", "k_adjoint_pair<{t}>"]
 # the library's default data movement of each row's kernel when untuned
-ROW_DEFAULT_VARIANT = {"A9 adjoint of z=a*b": 4, "A9 adjoint of z=a*b+c*d": 14}
+ROW_DEFAULT_VARIANT = {"A9 adjoint of z=a*b": 4, "A9 adjoint of z=a*b+c*d": 15}
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of a
 # kernel on a 32^4 lattice (1,048,576 sites; the batch row: its 64 fixed
@@ -134,7 +134,7 @@ def row_launches(r, tuned_variant):
         return r.name, 1, r.nbytes
     tree, math, prec, adj = ROW_TREE[r.name]
     v = tuned_variant if tuned_variant is not None else ROW_DEFAULT_VARIANT.get(r.name, 1)
-    if adj and v == 14:   # both products in one launch, dL/dZ read from HBM once
+    if adj and v == 15:   # both products in one launch, dL/dZ read from HBM once
         return "k_adjoint_pair_sum<%s>" % T_MM, 1, r.nbytes
     if adj and v >= 10:
         return ADJ_KERNEL[v - 10].format(t=T_MM, m="MathDF"), 2, B_ADJ_MM * r.sites

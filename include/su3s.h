@@ -431,9 +431,9 @@ int su3s_eval_adjoint(const su3s_expr* e, const su3s_field* grad_out, su3s_field
  * (a, b, grad_out -> dA, dB) and (c, d, grad_out -> dC, dD), which read
  * grad_out twice but hold the operands of one product at a time (two launches,
  * or one launch of both for a*b + c*d), and keeps the fastest form for later
- * calls (a split choice is reported as
- * *variant = 10 + the halves' data-movement variant).  Untuned calls of such
- * trees run split. */
+ * calls (two launches are reported as
+ * *variant = 10 + the halves' data-movement variant, one launch as 15).  Untuned
+ * calls of such trees run split. */
 int su3s_tune_adjoint(const su3s_expr* e, const su3s_field* grad_out, su3s_field* const* grad_leaves,
                       int nleaves, int math, void* stream, int* threads, int* blocks_per_sm,
                       int* variant, float* best_ms);

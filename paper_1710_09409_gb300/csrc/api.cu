@@ -1234,24 +1234,30 @@ static cudaError_t launch_planned(const EvalEntry* ent, const GParams& p, bool t
   return L.fn(&p, L.grid, L.block, st);
 }
 
-// The two products of a split reverse mode.  Both in one launch (kSplitSum)
-// needs the same kernel for both, staged fields, no other pipeline preferred
-// and two units for every warp that a product gets (one block of 8 warps on half
-// the SMs).  18^4 (1.35 units per warp of the chip): 43.8 us in two launches,
-// 30.9 in one.  16^4 (0.84) stays below the line: the two launches' smaller
-// blocks spread its tiles over more SMs (24.7 us).
-static cudaError_t launch_split(const SplitAdjoint& sp, int mode, cudaStream_t st) {
+// Whether the two products of a split reverse mode can run in one launch: the
+// same kernel for both, staged fields, no other pipeline preferred and two units
+// for every warp that a product gets (one block of 8 warps on half the SMs).
+// 18^4 (1.35 units per warp of the chip): 43.8 us in two launches, 30.9 in one.
+// 16^4 (0.84) stays below the line: the two launches' smaller blocks spread its
+// tiles over more SMs (24.7 us).
+static bool one_launch(const SplitAdjoint& sp) {
   const EvalEntry* e = sp.ent[0];
   const int pref = g_pipeline_pref.load(std::memory_order_relaxed);
   const int64_t nvec = sp.p[0].k.nvec, units = (nvec / 32 + 1) / 2;
   const int wpb = kSumThreads / 32, nmu = sp.p[0].k.nmu;
-  if (mode == kSplitSum && e->sum_fn && sp.ent[1] == e && sp.tma[0] && sp.tma[1] && nvec % 32 == 0 &&
-      (pref < 0 || pref == 4) && units * nmu >= (int64_t)wpb * sm_count()) {
+  return e->sum_fn && sp.ent[1] == e && sp.tma[0] && sp.tma[1] && nvec % 32 == 0 &&
+         (pref < 0 || pref == 4) && units * nmu >= (int64_t)wpb * sm_count();
+}
+
+// The two products of a split reverse mode; kSplitSum: in one launch where that
+// can be.
+static cudaError_t launch_split(const SplitAdjoint& sp, int mode, cudaStream_t st) {
+  if (mode == kSplitSum && one_launch(sp)) {
     GParamsSum both;
     both.half[0] = sp.p[0];
     both.half[1] = sp.p[1];
-    const int nb = pair_sum_blocks(sm_count(), nmu);
-    return e->sum_fn(&both, dim3((unsigned)nb, (unsigned)nmu, 1), dim3(kSumThreads, 1, 1), st);
+    const int nmu = sp.p[0].k.nmu, nb = pair_sum_blocks(sm_count(), nmu);
+    return sp.ent[0]->sum_fn(&both, dim3((unsigned)nb, (unsigned)nmu, 1), dim3(kSumThreads, 1, 1), st);
   }
   cudaError_t ce = launch_planned(sp.ent[0], sp.p[0], sp.tma[0], st);
   if (ce == cudaSuccess) ce = launch_planned(sp.ent[1], sp.p[1], sp.tma[1], st);
@@ -1339,9 +1345,9 @@ SU3S_EXPORT int su3s_tune_adjoint(const su3s_expr* e, const su3s_field* gout,
     if (!rc && sp.ent[1] != sp.ent[0])
       rc = tune_entry(sp.ent[1], &sp.p[1], p.k.nvec, p.k.nmu, sp.tma[1], st, nullptr, nullptr,
                       nullptr, &ms_half);
-    float ms_split = 0.f, ms_sum = 0.f;
+    float ms_split = 0.f, ms_sum = 1e30f;   // the one-launch form only where it runs
     if (!rc) rc = time_split(sp, kSplit, st, &ms_split);
-    if (!rc) rc = time_split(sp, kSplitSum, st, &ms_sum);
+    if (!rc && one_launch(sp)) rc = time_split(sp, kSplitSum, st, &ms_sum);
     if (rc) return rc;
     const bool split = ms_split < ms || ms_sum < ms, sum = ms_sum < ms_split;
     {
@@ -1351,7 +1357,7 @@ SU3S_EXPORT int su3s_tune_adjoint(const su3s_expr* e, const su3s_field* gout,
     if (split) {
       th = sum ? kSumThreads : th2;
       bps = sum ? 1 : bps2;
-      var = 10 + (sum ? 4 : var2);
+      var = 10 + (sum ? 5 : var2);
       ms = sum ? ms_sum : ms_split;
     }
   }
