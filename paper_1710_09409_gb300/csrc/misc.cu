@@ -222,9 +222,31 @@ __device__ __forceinline__ double row_norm2(const double* a) {
   return n;
 }
 
+// 1/sqrt(n) as y (1 + g): y the hardware's approximation cut to its leading word
+// (21 bits, so that y^2 is exact), e = 1 - n y^2, and g the series of
+// (1 - e)^(-1/2) - 1, exact to e^3 < 2^-56.  Kept in two parts, the factor enters
+// what it scales with one rounding.  1/n = y^2 / (1 - e).
+struct Rsqrt {
+  double y, g, w, e;   // w = y^2
+  __device__ __forceinline__ explicit Rsqrt(double n) {
+    double a;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(a) : "d"(n));
+    y = __hiloint2double(__double2hiint(a), 0);
+    w = y * y;
+    e = fma(-n, w, 1.0);
+    g = e * fma(e, 0.375, 0.5);
+  }
+  __device__ __forceinline__ double value() const { return fma(y, g, y); }
+  __device__ __forceinline__ double inverse() const { return fma(w, fma(e, e, e), w); }
+  // (t + h) / sqrt(n), q = t + h rounded
+  __device__ __forceinline__ double scale(double t, double h, double q) const {
+    return fma(t, y, y * fma(q, g, h));
+  }
+};
+
 // The same projection with fewer FP64 operations: the FP64 pipe bounds the
 // kernel (90% busy; 2.59 M FP64 matrices: 1,989 us by the definition's sweeps with
-// FP64 atan2 and sincos, which stay for the cases below, 951 here).
+// FP64 atan2 and sincos, which stay for the cases below, 952 here).
 // Row 1 takes a second sweep only where the first took out a sixteenth or more
 // of what it left (in norm squared): else one sweep leaves no more of row 0 than
 // its own rounding, as two do.  Of row 2 only a phase is free: orthonormal to
@@ -236,26 +258,28 @@ __device__ __forceinline__ double row_norm2(const double* a) {
 // signs of d), rounded to multiples of 2^-22 (its square is then exact in FP64)
 // and refined by one step on q^3 d/|d| = 1: with q^3 d/|d| = 1 + z, |z| < 1e-6,
 // q (1 - z/3 + 2/9 z^2) is exact to z^3 < 1e-18.  d/|d| is brought back to the
-// unit circle and q kept in two parts until the rows' norms are in it, as what q
-// rounds by is an error of all rows.  rms error against extended precision and,
-// in brackets, the definition's in FP64: projected matrices rounded to FP32
-// 4.22e-17 (4.31e-17), Gaussian 6.02e-17 (6.34e-17), projected matrices with
-// noise of 1e-3 4.69e-17 (4.48e-17).
+// unit circle, and q and the norms' reciprocal roots kept in two parts until they
+// are one factor of a row, as what such a factor rounds by is an error of the whole
+// row.  rms error against extended precision and, in brackets, the definition's in
+// FP64: projected matrices 3.40e-17 (3.45e-17), rounded to FP32 4.03e-17
+// (4.31e-17), with noise of 1e-6 to 1e-1 4.22 to 4.28e-17 (4.48 to 4.52e-17),
+// Gaussian 5.88e-17 (6.56e-17).  With rounded reciprocal roots noisy matrices had
+// 4.69e-17, in the same time (951 us).
 // Returns false where a norm is NaN, zero, or so large or small that it could
 // overflow or underflow here and not in the definition.
 __device__ __forceinline__ bool reunit_fast(double* r) {
   double* a = r;  // rows 0 and 1, not normalised until the end
   double* b = r + 6;
   const double n0 = row_norm2(a);
-  const double inv0 = rsqrt(n0);
-  const double rn0 = inv0 * inv0;
+  const Rsqrt s0(n0);
+  const double rn0 = s0.inverse();
   const double part = project_out(a, rn0, b);
   double n1 = row_norm2(b);
   if (part > n1 * 0.0625) {
     project_out(a, rn0, b);
     n1 = row_norm2(b);
   }
-  const double inv1 = rsqrt(n1);
+  const Rsqrt s1(n1);
   // x = a x b; d = sum_j x_j row2_j
   double x[6], dr = 0.0, di = 0.0;
 #pragma unroll
@@ -269,7 +293,7 @@ __device__ __forceinline__ bool reunit_fast(double* r) {
     di = fma(x[2 * j], r[12 + 2 * j + 1], fma(x[2 * j + 1], r[12 + 2 * j], di));
   }
   const double nd = fma(dr, dr, di * di);
-  const double invd = rsqrt(nd);
+  const double invd = Rsqrt(nd).value();
   if (!(n0 > 0x1p-200 && n0 < 0x1p200 && n1 > 0x1p-200 && n1 < 0x1p200 && nd > 0x1p-800 &&
         nd < 0x1p800))
     return false;
@@ -290,14 +314,14 @@ __device__ __forceinline__ bool reunit_fast(double* r) {
   const double hr = fma(tr, zr, -(ti * zi)), hi = fma(tr, zi, ti * zr);  // q = t + h
   const double qr = tr + hr, qi = ti + hi;
   // rows 0, 1: q over the norms, times the rows; row 2: e^{i alpha} q conj(x) /
-  // |x|, the conjugate of x/|x| times conj(e^{i alpha} q) (its norm taken with q
-  // as for rows 0, 1 costs 0.2e-17 of row 2's error)
-  const double inv2 = rsqrt(row_norm2(x));
-  const double pr = fma(er, qr, -(ei * qi)), pi = -fma(er, qi, ei * qr);
-  const double q0r = fma(tr, inv0, hr * inv0), q0i = fma(ti, inv0, hi * inv0);
-  const double q1r = fma(tr, inv1, hr * inv1), q1i = fma(ti, inv1, hi * inv1);
-#pragma unroll
-  for (int j = 0; j < 6; ++j) x[j] *= inv2;
+  // |x|, the conjugate of x times conj(e^{i alpha} q) over its norm
+  const Rsqrt s2(row_norm2(x));
+  const double yg = s2.y * s2.g;
+  double pr = fma(er, qr, -(ei * qi)), pi = -fma(er, qi, ei * qr);
+  pr = fma(pr, s2.y, pr * yg);
+  pi = fma(pi, s2.y, pi * yg);
+  const double q0r = s0.scale(tr, hr, qr), q0i = s0.scale(ti, hi, qi);
+  const double q1r = s1.scale(tr, hr, qr), q1i = s1.scale(ti, hi, qi);
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     zmul(r[2 * j], r[2 * j + 1], a[2 * j], a[2 * j + 1], q0r, q0i);
