@@ -236,7 +236,7 @@ struct Rsqrt {
     e = fma(-n, w, 1.0);
     g = e * fma(e, 0.375, 0.5);
   }
-  __device__ __forceinline__ double value() const { return fma(y, g, y); }
+  __device__ __forceinline__ double near() const { return fma(0.5 * y, e, y); }   // to e^2
   __device__ __forceinline__ double inverse() const { return fma(w, fma(e, e, e), w); }
   // (t + h) / sqrt(n), q = t + h rounded
   __device__ __forceinline__ double scale(double t, double h, double q) const {
@@ -293,7 +293,7 @@ __device__ __forceinline__ bool reunit_fast(double* r) {
     di = fma(x[2 * j], r[12 + 2 * j + 1], fma(x[2 * j + 1], r[12 + 2 * j], di));
   }
   const double nd = fma(dr, dr, di * di);
-  const double invd = Rsqrt(nd).value();
+  const double invd = Rsqrt(nd).near();   // |d|'s rest goes with the step to the unit circle
   if (!(n0 > 0x1p-200 && n0 < 0x1p200 && n1 > 0x1p-200 && n1 < 0x1p200 && nd > 0x1p-800 &&
         nd < 0x1p800))
     return false;
