@@ -146,8 +146,8 @@ __device__ __forceinline__ void load_obj(const FieldDesc& f, int64_t s, int mu, 
 }
 
 // Plain loads: a linear last term's leaf is read after the product in the pair
-// arithmetic, where its registers are free by then ((a*b)*c + s*d at 48^4: 959 us
-// with the term in pairs, 1,111 with the leaf read first, 941 after); in fixed
+// arithmetic, where its registers are free by then ((a*b)*c + s*d at 48^4: 957 us
+// with the term in pairs, 1,111 with the leaf read first, 945 after); in fixed
 // point it is read first (32^4: 198 us against 214).
 template <class Tree, class M>
 struct LateTail {

@@ -17,16 +17,6 @@ struct LatGeo {
   int64_t V;
 };
 
-// Site of s + shift e_dim (periodic); shift in (-L, L).  Volumes are below
-// 2^31, so the coordinate arithmetic is 32-bit.
-__device__ __forceinline__ int64_t shift_site(const LatGeo& g, int64_t s, int dim, int shift) {
-  const uint32_t st = (uint32_t)g.stride[dim], L = (uint32_t)g.L[dim];
-  const int32_t c = (int32_t)(((uint32_t)s / st) % L);
-  int32_t c2 = c + shift;
-  c2 = c2 >= (int32_t)L ? c2 - (int32_t)L : (c2 < 0 ? c2 + (int32_t)L : c2);
-  return s + (int64_t)(c2 - c) * st;
-}
-
 // FP64 object (W reals) of field f at site s, link mu, through the read-only
 // cache, in the arithmetic M.
 // g is the site's range guard (largest input high word, see dev_math.cuh).
@@ -66,8 +56,9 @@ __device__ __forceinline__ void load_link(const FieldDesc& f, int64_t s, int mu,
   M::template normalize_obj<18>(out);
 }
 
-// Site of s + shift e_mu for a runtime direction (the geometry is selected,
-// not indexed, so it stays in registers).
+// Site of s + shift e_mu (periodic) for a runtime direction; shift in (-L, L).
+// The geometry is selected, not indexed, so it stays in registers; volumes are
+// below 2^31, so the coordinate arithmetic is 32-bit.
 __device__ __forceinline__ int64_t shift_site_rt(const LatGeo& g, int64_t s, int mu, int shift) {
   const uint32_t st = (uint32_t)(mu == 0 ? g.stride[0] : mu == 1 ? g.stride[1] : mu == 2 ? g.stride[2] : g.stride[3]);
   const uint32_t L = (uint32_t)(mu == 0 ? g.L[0] : mu == 1 ? g.L[1] : mu == 2 ? g.L[2] : g.L[3]);

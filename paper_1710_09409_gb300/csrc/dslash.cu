@@ -630,8 +630,8 @@ static cudaError_t launch_dslash(const su3s_field* dest, const su3s_field* U, co
   // 32 waves: each wave of a grid-stride loop lets its blocks drift apart, new
   // blocks start in the order of the sites, so that the neighbours of those in
   // flight stay in the L2 cache.  Fixed point: one wave 2,094 us, four 2,086,
-  // eight 2,064, 32 1,985, one site per thread 2,044 at 32^3 x 64; 156 against
-  // 145 at 16^3 x 32.  FP64 4,037 -> 4,002.
+  // eight 2,064, 32 1,985, one site per thread 2,044 at 32^3 x 64; at 16^3 x 32
+  // one wave 156, 32 waves 145.  FP64 at 32^3 x 64: one wave 4,037, 32 waves 4,002.
   const cudaError_t e = dslash_grid((const void*)k_dslash<M>, smem, g.V, 32, &grid);
   if (e != cudaSuccess) return e;
   k_dslash<M><<<grid, kDslashThreads, smem, st>>>(dest->desc, U->desc, psi->desc, g);

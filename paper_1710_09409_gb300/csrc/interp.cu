@@ -8,7 +8,8 @@
 // operands into fixed-size arrays (their widths are known per operation), so
 // the arithmetic runs on registers, and writes its result back.  The host
 // sizes the shared memory to the registers the program uses: leaves are
-// loaded at their first use and every register is freed after its last.
+// loaded at their first use and every register is freed after the last operation
+// that reads it (interp_prog.h).
 #include <string.h>
 
 #include <mutex>

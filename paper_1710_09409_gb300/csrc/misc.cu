@@ -245,8 +245,8 @@ struct Rsqrt {
 };
 
 // The same projection with fewer FP64 operations: the FP64 pipe bounds the
-// kernel (90% busy; 2.59 M FP64 matrices: 1,989 us by the definition's sweeps with
-// FP64 atan2 and sincos, which stay for the cases below, 952 here).
+// kernel (91% busy; 2.59 M FP64 matrices: 1,989 us by the definition's sweeps with
+// FP64 atan2 and sincos, which stay for the cases below, 948 here).
 // Row 1 takes a second sweep only where the first took out a sixteenth or more
 // of what it left (in norm squared): else one sweep leaves no more of row 0 than
 // its own rounding, as two do.  Of row 2 only a phase is free: orthonormal to
@@ -261,7 +261,7 @@ struct Rsqrt {
 // unit circle, and q and the norms' reciprocal roots kept in two parts until they
 // are one factor of a row, as what such a factor rounds by is an error of the whole
 // row.  rms error against extended precision and, in brackets, the definition's in
-// FP64: projected matrices 3.40e-17 (3.45e-17), rounded to FP32 4.03e-17
+// FP64: projected matrices 3.40e-17 (3.45e-17), rounded to FP32 4.08e-17
 // (4.31e-17), with noise of 1e-6 to 1e-1 4.22 to 4.28e-17 (4.48 to 4.52e-17),
 // Gaussian 5.88e-17 (6.56e-17).  With rounded reciprocal roots noisy matrices had
 // 4.69e-17, in the same time (951 us).

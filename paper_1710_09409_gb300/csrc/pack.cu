@@ -16,12 +16,12 @@ namespace su3s {
 // that neither side has bank conflicts): one side of the copy walks the host
 // array's run of the tile, the other whole 32-site rows of an element, and both
 // are full 128-byte lines.  HBM-bound.  Measured, FP64 links of 23x25x24x47
-// (1.49 GB of canonical array and field): pack 379 -> 249 us, unpack 231 ->
-// 240 us against one element per thread in host order (16-byte pieces of the
-// field at a time, four 64-bit divisions each).
+// (747 MB of canonical array and field): pack 379 -> 127 us, unpack 231 -> 119 us
+// against one element per thread in host order (16-byte pieces of the field at a
+// time, four 64-bit divisions each).
 
 // One host element and its stored form.  H: the host array's element, moved as
-// VEC pieces when the array is not aligned to it.
+// two doubles when the array is not aligned to it.
 template <int PREC>
 struct CanonElem {  // canonical complex <-> stored complex
   using H = double2;

@@ -315,8 +315,11 @@ static cudaError_t launch_hop(const su3s_field* dest, const su3s_field* U, const
   // 32^3 x 64, one wave, four, 32: pair arithmetic on matrices 1,086, 998, 955 us;
   // fixed point on vectors 604, 548, 536, on matrices 1,361, 1,358, 1,345; FP64
   // 1,212, 1,177, 1,175 and 3,700, 3,602, 3,579.  Fixed-point matrices below eight
-  // waves keep one: 94.8 us against 96.8 at 16^3 x 32, 3.4 waves (230 against
-  // 228 at 8.5).
+  // waves keep one; there the two come out alike.  One wave against 32 at 20 sizes:
+  // within 1% at nine, one faster at eight (14^3 x 28 51.5 / 52.9 us, 16^3 x 32 94.4 /
+  // 96.5, 20^3 x 30 164.6 / 169.9, 20^3 x 40 212 / 219 and others, 1.5 to 3%), 32 at
+  // three (18^3 x 30 130 / 123, 18^3 x 36 155 / 146, 24^4 229 / 227): how full the
+  // last round of blocks is decides, not the number of waves.
   const int64_t wave = (int64_t)(per_sm > 0 ? per_sm : 1) * sm_count();
   const int64_t need = (g.V + 127) / 128;
   const int64_t nb = M::kScaled && KIND == KM && need < 8 * wave ? wave : 32 * wave;
